@@ -164,15 +164,14 @@ typedef struct hough_tracks {
 
 /*
  * Launch shape of the find kernel; 0 in a field means "library default".
- * All fields 0: the first shape that fits of 3 CTAs of 256 threads per SM,
- * 2 of 512 and 1 of 1024, with 32-word-row tiles (else one CTA of 512
- * threads with the largest tile that fits); when that is 3 CTAs of 256
- * threads, a batch of more than 250 hits per window on average runs in 2
- * CTAs of 512 instead (its candidate lists need the larger CTAs' shared
- * memory).  hough_get_launch returns the first choice.
+ * All fields 0: as many CTAs per SM as fit, up to four, with 32-word-row
+ * tiles: four of 128 threads, three or two of 256, one of 512; batches of few
+ * windows (up to two per SM), and of few or many hits per window where two
+ * CTAs fit, run in CTAs of another size (chosen per batch).
+ * hough_get_launch returns the first choice.
  */
 typedef struct hough_launch {
-    int32_t threads;      /* threads per CTA: 256, 512 or 1024                     */
+    int32_t threads;      /* threads per CTA: 128, 256, 512 or 1024                */
     int32_t word_rows;    /* word rows of the shared accumulator tile: 32, 64 or 128   */
     int32_t hit_stage;    /* hits held in shared memory per stage (multiple of 256)  */
     int32_t ctas_per_sm;  /* resident CTAs per SM (1..4); capped by occupancy       */

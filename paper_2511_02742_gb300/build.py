@@ -17,7 +17,8 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 SRC = os.path.join(PKG, "csrc", "hough_api.cu")
 SERVER_SRC = os.path.join(PKG, "csrc", "hough_server.cpp")
-FIND_SRCS = [os.path.join(PKG, "csrc", "hough_find.cu"), os.path.join(PKG, "csrc", "hough_find_fp64.cu")]
+FIND_SRCS = [os.path.join(PKG, "csrc", f"hough_find{k}.cu")
+             for k in ("", "_128", "_256", "_512", "_1024", "_fp64")]
 UNITS = [SRC, *FIND_SRCS, SERVER_SRC]
 DEPS = [*UNITS, os.path.join(PKG, "csrc", "hough_kernels.cuh"),
         os.path.join(PKG, "csrc", "hough_encode.cuh"),

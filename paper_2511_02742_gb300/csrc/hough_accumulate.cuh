@@ -8,11 +8,6 @@
 
 namespace hk {
 
-__device__ __forceinline__ void red_add_shared(unsigned addr, unsigned v)
-{
-    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(v));
-}
-
 // Every staged hit votes once in each of the tile's rows.  No vote needs its
 // returned count here (nothing is listed), so the votes are reductions.
 // FAST: every valid hit votes in range and the tile has no row past n_theta.
@@ -145,7 +140,7 @@ __device__ void acc_window(const KParams &p, long long beg, int H, uint32_t *acc
     const int acc_words4 = (WR * p.n_rho) >> 2;
     int nv = 0;
     if (single)
-        nv = stage_hits(p, beg, H, stage, wtot, ws);
+        nv = stage_hits<AnyShape>(p, beg, H, stage, wtot, ws);
     bool oor = false;
     for (int tile = 0; tile < n_tiles; ++tile) {
         const int t0 = tile * R;
@@ -161,7 +156,7 @@ __device__ void acc_window(const KParams &p, long long beg, int H, uint32_t *acc
         } else {
             for (long long s0 = 0; s0 < H; s0 += p.hit_stage) {
                 const int n = (int)min((long long)p.hit_stage, (long long)H - s0);
-                const int ns = stage_hits(p, beg + s0, n, stage, wtot, ws);
+                const int ns = stage_hits<AnyShape>(p, beg + s0, n, stage, wtot, ws);
                 acc_vote_tile<P, false>(p, acc, stage, ns, t0, oor);
                 __syncthreads();
             }
@@ -180,7 +175,7 @@ __global__ void __launch_bounds__(1024, 1) accumulate_kernel(KParams p)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ WinScalars ws;
-    __shared__ int wtot[32];
+    __shared__ int wtot[64];
     uint32_t *acc = reinterpret_cast<uint32_t *>(smem);
     int2 *stage = reinterpret_cast<int2 *>(smem + align_up((size_t)p.word_rows * p.n_rho * 4, 16));
     for (long long w = blockIdx.x; w < p.n_windows; w += gridDim.x) {

@@ -211,45 +211,55 @@ int next_pow2(int x)
     return n;
 }
 
-// Candidate-list entries: whatever shared memory the tile leaves, up to what
-// lists holding every counter of the tile and of the carried row need.
-// Returns -1 when fewer than max(1024, threads + 64 per warp) would fit: a
-// list that overflows only sends its tile to the direct test, but every
-// warp needs at least two column slots per lane and the check needs one
-// gathered entry per thread.
-int cl_entries_for(const hough_ctx *ctx, int word_rows, int hit_stage, int ctas, int threads)
+// Top-k region of a context's windows: the kept peaks, rounded up.
+int kept_region(const hough_ctx *ctx)
 {
-    const int nw = threads / 32;
-    // per CTA the SM also reserves 1 KB and holds the kernel's static shared
-    // variables (kStaticSmemReserve covers them): `ctas` CTAs must fit
-    const size_t budget = std::min(ctx->smem_optin,
-                                   ctx->smem_per_sm / (size_t)ctas - 1024 - kStaticSmemReserve);
-    const int nb = tile_bins(ctx, word_rows);
-    hk::SmemLayout L0 = hk::smem_layout(word_rows, hit_stage, nb, 0, nw);
-    long long room = L0.total < budget ? (long long)((budget - L0.total) / 4) : 0;
-    // lists able to hold every counter of the tile and of the carried row in
-    // their columns, plus the gathered-entry sixth
-    const long long need = std::max<long long>(1024, threads + 64LL * nw);
-    const long long worst = (4LL * word_rows * nb + nb) * 12 / 5 + threads;
-    long long n = std::min(room, std::max(worst, need));
-    n -= n % (4 * nw);
-    if (n < need)
-        return -1;
-    return (int)n;
+    return std::max(32, next_pow2(std::max(1, ctx->th.max_peaks)));
+}
+
+// Shared memory of the find kernel's tile, which the association also uses
+// for its counts and slots, one of each per warp and category.
+size_t acc_bytes_for(const hough_ctx *ctx, int word_rows, int threads)
+{
+    return hk::align_up(std::max(hk::tile_words(word_rows, tile_bins(ctx, word_rows)) * 4,
+                                 (size_t)(threads / 32) * (ctx->th.max_peaks + 2) * 8),
+                        16);
+}
+
+size_t find_smem(const hough_ctx *ctx, int word_rows, int hit_stage, int threads)
+{
+    return hk::smem_layout(acc_bytes_for(ctx, word_rows, threads), hit_stage,
+                           tile_bins(ctx, word_rows), kept_region(ctx), threads / 32)
+        .total;
+}
+
+// Whether `ctas` CTAs of this much dynamic shared memory fit on an SM: per
+// CTA the SM also reserves 1 KB and holds the kernel's static shared
+// variables (kStaticSmemReserve covers them).
+bool smem_fits(const hough_ctx *ctx, size_t smem, int ctas)
+{
+    return smem <= std::min(ctx->smem_optin,
+                            ctx->smem_per_sm / (size_t)ctas - 1024 - kStaticSmemReserve);
 }
 
 // Fill in defaults and check a launch shape against the device limits.
 int resolve_launch(const hough_ctx *ctx, const hough_launch &in, hough_launch &out, size_t &smem)
 {
     hough_launch l = in;
-    // Fully default: the first of these that fits, all with 32-word-row
-    // tiles: three CTAs of 256 threads per SM, two of 512 (several CTAs per
-    // SM overlap one CTA's barriers with the others' votes, and small CTAs
-    // wait less at each barrier), one of 1024; else one CTA of 512 threads
-    // with the largest tile.
+    // Fully default: as many CTAs per SM as fit, up to four (windows on an SM
+    // overlap one another's barriers and latency), with tiles of 32 word
+    // rows.  The fewer fit, the more threads each has: every tile costs each
+    // warp a fixed share (its part of the scan, a partly filled test step, the
+    // barriers), so beside other windows small CTAs do less work per window
+    // (four of 128 threads against four of 256 at 512 x 512: 23 k against 35 k
+    // warp instructions per 70-hit window, 0.66 against 0.79 ms per 2e4), and
+    // alone on the SM they leave it idle.
     if (l.threads == 0 && l.word_rows == 0 && l.hit_stage == 0 && l.ctas_per_sm == 0) {
-        for (const hough_launch &c : {hough_launch{256, 32, 512, 3}, hough_launch{512, 32, 1024, 2},
-                                      hough_launch{1024, 32, 2048, 1}})
+        for (const hough_launch &c :
+             {hough_launch{128, 32, 1024, 4}, hough_launch{128, 32, 512, 4},
+              hough_launch{256, 32, 1024, 3}, hough_launch{256, 32, 512, 3},
+              hough_launch{256, 32, 2048, 2}, hough_launch{256, 32, 1024, 2},
+              hough_launch{512, 32, 2048, 1}})
             if (resolve_launch(ctx, c, out, smem) == HOUGH_OK)
                 return HOUGH_OK;
     }
@@ -262,18 +272,14 @@ int resolve_launch(const hough_ctx *ctx, const hough_launch &in, hough_launch &o
     if (l.word_rows == 0) {
         // the largest tile that fits, as long as 16-bit tiles do not pass n_theta
         l.word_rows = 32;
-        for (int wr : {128, 64}) {
-            hk::SmemLayout L = hk::smem_layout(wr, l.hit_stage, tile_bins(ctx, wr), 4096,
-                                               l.threads / 32);
-            if ((L.total + 1024 + kStaticSmemReserve) * (size_t)l.ctas_per_sm <= ctx->smem_per_sm &&
-                L.total <= ctx->smem_optin &&
-                ctx->n_theta >= 2 * wr) {
+        for (int wr : {128, 64})
+            if (ctx->n_theta >= 2 * wr &&
+                smem_fits(ctx, find_smem(ctx, wr, l.hit_stage, l.threads), l.ctas_per_sm)) {
                 l.word_rows = wr;
                 break;
             }
-        }
     }
-    if (!(l.threads == 256 || l.threads == 512 || l.threads == 1024))
+    if (!(l.threads == 128 || l.threads == 256 || l.threads == 512 || l.threads == 1024))
         return HOUGH_ERR_INVALID_ARG;
     if (!(l.word_rows == 32 || l.word_rows == 64 || l.word_rows == 128))
         return HOUGH_ERR_INVALID_ARG;
@@ -281,48 +287,47 @@ int resolve_launch(const hough_ctx *ctx, const hough_launch &in, hough_launch &o
         return HOUGH_ERR_INVALID_ARG;
     if (l.ctas_per_sm < 1 || l.ctas_per_sm > 4)
         return HOUGH_ERR_INVALID_ARG;
-    const int cl = cl_entries_for(ctx, l.word_rows, l.hit_stage, l.ctas_per_sm, l.threads);
-    if (cl < 0)
-        return HOUGH_ERR_UNSUPPORTED_SHAPE;    // no room for useful candidate lists
-    // association keeps one count per warp and category in the tile or in
-    // the list area
-    const long long cat_counts = (long long)(l.threads / 32) * (ctx->th.max_peaks + 2);
-    if (cat_counts > (long long)l.word_rows * tile_bins(ctx, l.word_rows) && cat_counts > cl)
-        return HOUGH_ERR_UNSUPPORTED_SHAPE;
-    hk::SmemLayout L = hk::smem_layout(l.word_rows, l.hit_stage, tile_bins(ctx, l.word_rows), cl,
-                                       l.threads / 32);
-    if (L.total > ctx->smem_optin)
+    const size_t need = find_smem(ctx, l.word_rows, l.hit_stage, l.threads);
+    if (!smem_fits(ctx, need, l.ctas_per_sm))
         return HOUGH_ERR_UNSUPPORTED_SHAPE;
     out = l;
-    smem = L.total;
+    smem = need;
     return HOUGH_OK;
 }
 
-// The shape a find of n_windows windows and n_hits hits runs in: `base`, or,
-// when the shape was left to the library (automatic) and its default is
-// three 256-thread CTAs per SM, two 512-thread CTAs per SM for windows of
-// more than kHeavyWindowHits hits on average.  Heavier windows list more
-// candidate bins per tile than the small CTAs' shared memory holds.  Where
-// the shapes cross depends on the spread of window sizes as well as the
-// mean: Poisson mixes of tracks at 71 / 143 / 199 / 256 / 313 / 427 hits per
-// window ran 0.71 / 0.78 / 0.83 / 0.87 / 0.99 / 1.16 times as long in three
-// 256-thread CTAs as in two 512-thread ones, and a uniform mix of 1 to 40
-// tracks (295 hits, with a long tail) 1.24 times.
-constexpr int64_t kHeavyWindowHits = 250;
-
 }  // namespace
+
+// The shape a find of n_windows windows and n_hits hits runs in: `base`, or,
+// when the shape was left to the library (automatic), one of other CTA sizes:
+//  - up to one window per SM: one CTA of 512 threads, of 1024 for more than
+//    kHeavyWindowHits hits per window on average (100 windows of 290 hits at
+//    512 x 512: 91, 72, 54 and 51 us with 128, 256, 512 and 1024 threads; one
+//    window of 142 hits 29, 27, 26 and 27 us);
+//  - up to two: two CTAs of 256 (300 windows of 290 hits: 103 and 80 us with
+//    128 and 256 threads);
+//  - where two CTAs fit on an SM: 128 threads each up to kLightWindowHits hits
+//    per window, 512 above kHeavyWindowHits (3000 windows at 1024 x 1024, 128
+//    / 256 / 512 threads: 142 hits 0.47 / 0.51 / 0.50 ms, 285 hits 0.73 / 0.73 /
+//    0.72, 570 hits 1.35 / 1.23 / 1.11, 960 hits 2.09 / 1.80 / 1.59).
+constexpr int64_t kLightWindowHits = 200, kHeavyWindowHits = 280;
 
 hough_launch launch_for(const hough_ctx *ctx, const hough_launch &base, bool automatic,
                         int64_t n_hits, int64_t n_windows)
 {
-    if (!automatic || n_windows <= 0 || base.threads != 256 || base.ctas_per_sm != 3 ||
-        n_hits <= kHeavyWindowHits * n_windows)
+    if (!automatic || n_windows <= 0)
         return base;
+    const bool heavy = n_hits > kHeavyWindowHits * n_windows;
+    const bool light = n_hits <= kLightWindowHits * n_windows;
+    hough_launch want = base;
+    if (n_windows <= ctx->num_sms)
+        want = hough_launch{heavy ? 1024 : 512, 32, 2048, 1};
+    else if (n_windows <= 2 * (int64_t)ctx->num_sms)
+        want = hough_launch{256, 32, 1024, 2};
+    else if (base.ctas_per_sm == 2 && (heavy || light))
+        want = hough_launch{heavy ? 512 : 128, 32, base.hit_stage, 2};
     hough_launch l{};
     size_t smem = 0;
-    if (resolve_launch(ctx, hough_launch{512, 32, 1024, 2}, l, smem) == HOUGH_OK)
-        return l;
-    return base;
+    return resolve_launch(ctx, want, l, smem) == HOUGH_OK ? l : base;
 }
 
 namespace {
@@ -401,19 +406,13 @@ hk::KParams make_params(const hough_ctx *ctx, const hough_hits *hits, const int6
     p.n_b = narrow ? tile_bins(ctx, l.word_rows) : ctx->n_rho;
     p.lo_tab = narrow && ctx->d_lo ? ctx->d_lo + (size_t)wi * 3 * ctx->lo_stride : nullptr;
     p.lo_stride = ctx->lo_stride;
-    p.nb_inv = (unsigned)(((1ull << 32) + (unsigned long long)p.n_b - 1) /
-                          (unsigned long long)p.n_b);
-    p.nrho_inv = (unsigned)(((1ull << 32) + (unsigned long long)ctx->n_rho - 1) /
-                            (unsigned long long)ctx->n_rho);
     p.hit_stage = l.hit_stage;
-    p.kp = std::max(32, next_pow2(std::max(1, ctx->th.max_peaks)));
-    // the list area, split into per-warp lists (a multiple of 32 entries),
-    // half of each being the warp's overflow area: a lane's column overflows
-    // when its word row is crossed by many more lines than the average row
-    const int cl = cl_entries_for(ctx, l.word_rows, l.hit_stage, l.ctas_per_sm, l.threads);
-    p.cl_total = cl;
-    p.seg_cl = (cl / (l.threads / 32)) & ~31;
-    p.seg_ovf = (p.seg_cl / 2) & ~31;
+    p.kp = kept_region(ctx);
+    while ((1 << p.tb) < ctx->n_theta)
+        ++p.tb;
+    while ((1 << p.bb) < ctx->n_rho)
+        ++p.bb;
+    p.acc_bytes = (unsigned)acc_bytes_for(ctx, l.word_rows, l.threads);
     return p;
 }
 
@@ -425,12 +424,20 @@ struct Prepared {
 
 // The find kernel of a context: fixed-point bins, or the FP64 variant.
 using FindKernel = void (*)(hk::KParams);
-// The find kernel for this context and CTA size.
-static FindKernel find_kernel_of(const hough_ctx *ctx, int threads)
+// The find kernel for this context and launch shape.
+static FindKernel find_kernel_of(const hough_ctx *ctx, const hough_launch &l)
 {
     if (ctx->th.flags & HOUGH_FLAG_FP64)
         return hk::find_kernel_fp64;
-    return threads <= 256 ? hk::find_kernel_256 : hk::find_kernel;
+    if (l.word_rows != 32)
+        return hk::find_kernel;
+    switch (l.threads) {
+    case 128: return hk::find_kernel_128;
+    case 256: return hk::find_kernel_256;
+    case 512: return hk::find_kernel_512;
+    case 1024: return hk::find_kernel_1024;
+    default: return hk::find_kernel;
+    }
 }
 
 // Resolve a launch shape, raise the kernel's shared-memory limit and size the
@@ -440,7 +447,7 @@ int prepare_find(hough_ctx *ctx, int64_t n_windows, const hough_launch &req, Pre
     int rc = resolve_launch(ctx, req, pr.l, pr.smem);
     if (rc != HOUGH_OK)
         return rc;
-    const FindKernel fk = find_kernel_of(ctx, pr.l.threads);
+    const FindKernel fk = find_kernel_of(ctx, pr.l);
     if (raise_smem_limit(reinterpret_cast<const void *>(fk), pr.smem) != HOUGH_OK)
         return HOUGH_ERR_CUDA;
     cudaFuncAttributes fa{};
@@ -461,7 +468,7 @@ int enqueue_find(hough_ctx *ctx, const hough_hits *hits, const int64_t *offsets,
                  unsigned int *counter, const Prepared &pr)
 {
     hk::KParams p = make_params(ctx, hits, offsets, n_windows, out, counter, pr.l);
-    find_kernel_of(ctx, pr.l.threads)<<<pr.grid, pr.l.threads, pr.smem, s>>>(p);
+    find_kernel_of(ctx, pr.l)<<<pr.grid, pr.l.threads, pr.smem, s>>>(p);
     if (cudaGetLastError() != cudaSuccess)
         return HOUGH_ERR_CUDA;
     ctx->launches += 1;
@@ -1392,7 +1399,7 @@ int hough_autotune(hough_ctx *ctx, const hough_hits *hits, const int64_t *window
         return fail(ctx, HOUGH_ERR_CUDA);
     hough_launch chosen = ctx->launch;
     float best_ms = 1e30f;
-    for (int threads : {256, 512, 1024})
+    for (int threads : {128, 256, 512, 1024})
         for (int wr : {32, 64, 128})
             for (int cps : {1, 2, 3, 4})
                 for (int hs : {1024, 2048}) {

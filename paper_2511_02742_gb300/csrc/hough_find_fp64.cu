@@ -7,7 +7,7 @@ namespace hk {
 // Any CTA size up to 1024 threads.
 __global__ void __launch_bounds__(1024, 1) find_kernel_fp64(KParams p)
 {
-    find_body<true>(p);
+    find_body<AnyShape, true>(p);
 }
 
 }  // namespace hk

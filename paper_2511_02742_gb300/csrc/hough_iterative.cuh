@@ -6,8 +6,8 @@
 //
 // One CTA per window (grid-stride).  The window's valid hits are staged in
 // shared memory with their window-local indices; every iteration runs the
-// theta tiles of the find kernel's vote loop (its narrowed tiles, vote_tile
-// with candidate listing switched off) and a block maximum over each tile's
+// theta tiles of the find kernel's vote loop (its narrowed tiles of 32 word
+// rows, stored without guard columns) and a block maximum over each tile's
 // counters, then marks the line's hits and compacts them out of the stage in
 // order.
 #pragma once
@@ -125,15 +125,13 @@ __device__ unsigned long long tile_best(const KParams &p, const uint32_t *acc, i
         const uint32_t wv = acc[f];
         if (!has_field<P>(wv, top))
             continue;
-        const int q = f >> 5;
-        const int g = (int)__umulhi((unsigned)q, p.nb_inv);
-        const int b = q - g * p.n_b + lo;                   // the tile stores bins lo ..
-        const int wr = g * 32 + (f & 31);
+        const int b = (f >> 5) + lo;                        // the tile stores bins lo ..
+        const int wr = f & 31;
 #pragma unroll
         for (int s = 0; s < P; ++s) {
             if (((wv >> (s * CW)) & MASK) != top)
                 continue;
-            const int t = t0 + s * p.word_rows + wr;
+            const int t = t0 + wr * P + s;
             const unsigned long long key = ((unsigned long long)top << 32) |
                                            (unsigned long long)(0xffffffffu -
                                                                 (((unsigned)t << 16) | (unsigned)b));
@@ -164,8 +162,7 @@ __device__ unsigned long long iter_best(const KParams &p, uint32_t *acc, const i
     const int32_t *lo_row = p.lo_tab ? p.lo_tab + lgP * p.lo_stride : nullptr;
     unsigned long long best = 0ull;
     int best_tile = n_tiles;
-    int cnt = 0;
-    const ListOvf none{&ws.n_sel, 0};
+    const unsigned acc0 = (unsigned)__cvta_generic_to_shared(acc);
     for (int i = threadIdx.x; i < (n_tiles + 31) / 32; i += blockDim.x)
         done[i] = 0u;
     __syncthreads();
@@ -198,9 +195,9 @@ __device__ unsigned long long iter_best(const KParams &p, uint32_t *acc, const i
             acc4[i] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
         if (p.in_range && t0 + R <= p.n_theta)
-            vote_tile<P, true>(p, acc, stage, nv, t0, lo, nullptr, 0, cnt, none, ws);
+            vote_tile<Shape<512, 32>, P, true>(p, acc0, 0u, stage, nv, t0, lo, ws);
         else
-            vote_tile<P, false>(p, acc, stage, nv, t0, lo, nullptr, 0, cnt, none, ws);
+            vote_tile<Shape<512, 32>, P, false>(p, acc0, 0u, stage, nv, t0, lo, ws);
         __syncthreads();
         const unsigned long long k = tile_best<P>(p, acc, t0, lo, red);
         if (threadIdx.x == 0) {
@@ -225,9 +222,8 @@ __global__ void __launch_bounds__(512, 1) iterative_kernel(IterParams q)
     __shared__ int taken;
     __shared__ int ub[HOUGH_MAX_THETA / 32];      // per-tile bounds (at most n_theta / 32 tiles)
     __shared__ unsigned done[HOUGH_MAX_THETA / 32 / 32];
-    KParams p = q.k;
-    p.T = 0x7fffffff;               // the vote loop lists nothing
-    const int T = q.k.T;
+    const KParams &p = q.k;
+    const int T = p.T;
     uint32_t *acc = reinterpret_cast<uint32_t *>(smem);
     int2 *stage = reinterpret_cast<int2 *>(smem + (size_t)p.word_rows * p.n_b * 4);
     int *sidx = reinterpret_cast<int *>(stage + p.hit_stage);

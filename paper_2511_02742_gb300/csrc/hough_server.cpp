@@ -8,7 +8,9 @@
 //   retire  -- a busy slot whose completion event has fired: complete its
 //              requests (their results are in their buffers already);
 //   admit   -- a free slot and a non-empty queue: take requests, oldest
-//              first, while the slot's window and hit capacity allows,
+//              first, while the slot's window and hit capacity allows
+//              (while another batch is on the GPU, fewer windows than SMs
+//              wait a moment for more),
 //              write the batch's window offsets (rebased) into the slot's
 //              pinned staging, then on the slot's stream copy them and each
 //              request's hits in, launch the find kernel, copy the results
@@ -41,6 +43,12 @@ size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // How long an idle worker polls the queue before it sleeps.
 constexpr int64_t kIdleSpinNs = 2'000'000;
+
+// How long a request may wait for others while a batch is on the GPU and the
+// queue holds fewer windows than the GPU has SMs: requests that come one
+// after the other are then served by few batches with a window per SM, not by
+// one batch (ten copies and a launch) each.  About the time of such a batch.
+constexpr int64_t kGatherNs = 60'000;
 
 int64_t now_ns()
 {
@@ -84,6 +92,7 @@ struct Pending {
     uint64_t ticket = 0;
     hough_request req{};
     int64_t n_hits = 0;
+    int64_t queued_ns = 0;
 };
 
 struct Slot {
@@ -194,7 +203,7 @@ int launch_slot(hough_server *s, Slot &sl)
     if (s->per_batch)
         s->ctx->launch = sl.W >= 2 * (int64_t)s->ctx->num_sms
                              ? launch_for(s->ctx, s->thr_launch, s->thr_auto, sl.H, sl.W)
-                             : s->lat_launch;
+                             : launch_for(s->ctx, s->lat_launch, true, sl.H, sl.W);
     int rc = hough_find(s->ctx, &hits, reinterpret_cast<const int64_t *>(sl.d_in + L.off), sl.W,
                         &t, sl.stream);
     if (rc != HOUGH_OK)
@@ -260,6 +269,21 @@ void complete_slot(hough_server *s, Slot &sl, int64_t t_done)
     s->cv_done.notify_all();
 }
 
+// Whether the queued requests should wait for others (lock held).
+bool gather(const hough_server *s)
+{
+    bool busy = false;
+    for (const Slot &sl : s->slots)
+        busy = busy || sl.busy;
+    if (!busy || s->stop || s->queue.empty())
+        return false;
+    int64_t windows = 0;
+    for (const Pending &p : s->queue)
+        if ((windows += p.req.n_windows) >= s->ctx->num_sms)
+            return false;
+    return now_ns() - s->queue.front().queued_ns < kGatherNs;
+}
+
 void worker_loop(hough_server *s)
 {
     cudaSetDevice(s->ctx->device);
@@ -283,7 +307,7 @@ void worker_loop(hough_server *s)
         }
         // admit
         for (Slot &sl : s->slots) {
-            if (sl.busy || s->queue.empty())
+            if (sl.busy || s->queue.empty() || gather(s))
                 continue;
             sl.reqs.clear();
             sl.win_base.clear();
@@ -396,12 +420,12 @@ int hough_server_create(hough_ctx *ctx, const hough_server_config *cfg, hough_se
     s->ctx = ctx;
     s->cfg = *cfg;
     s->max_peaks = ctx->th.max_peaks;
-    // the server's launch shape: as given, else chosen per batch: one CTA of
-    // 1024 threads per SM with 32-word-row tiles for small batches (they then
-    // spread over every SM, and each window has the most warps), the
-    // context's own shape (the library default, or what hough_set_launch or
-    // hough_autotune chose for the workload) for batches of at least two
-    // windows per SM
+    // the server's launch shape: as given, else chosen per batch: large CTAs,
+    // one or two per SM (launch_for), for batches of fewer than two windows
+    // per SM, so that they spread over every SM and each window has many
+    // warps; the context's own shape (the library's choice, or what
+    // hough_set_launch or hough_autotune chose for the workload) for larger
+    // ones
     s->saved_launch = ctx->launch;
     s->saved_auto = ctx->auto_launch;
     s->thr_auto = ctx->auto_launch;
@@ -512,6 +536,7 @@ int hough_server_submit(hough_server *s, const hough_request *req, uint64_t *tic
     p.n_hits = nh;
     if (p.req.arrival_ns == 0)
         p.req.arrival_ns = now_ns();
+    p.queued_ns = now_ns();
     s->queue.push_back(p);
     s->queued.fetch_add(1, std::memory_order_release);
     s->live.insert(p.ticket);
