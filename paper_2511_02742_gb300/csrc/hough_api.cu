@@ -998,35 +998,62 @@ int hough_find_iterative(hough_ctx *ctx, const hough_hits *hits, const int64_t *
         return fail(ctx, HOUGH_ERR_INVALID_ARG);
     if (n_windows == 0)
         return HOUGH_OK;
-    // 512 threads, tiles of 32 word rows beside the stage of hits and the
-    // kernel's static shared variables (small tiles let more of them be
+    // the windows of ordinary size: as many CTAs per SM as leave room for twice
+    // the average window's hits and a list of bins
+    cudaFuncAttributes fa{}, fb{};
+    if (cudaFuncGetAttributes(&fa, hk::iterative_kernel_128) != cudaSuccess ||
+        cudaFuncGetAttributes(&fb, hk::iterative_tiles_kernel) != cudaSuccess)
+        return fail(ctx, HOUGH_ERR_CUDA);
+    const int nb = tile_bins(ctx, 32);
+    const long long mean = hits->n_hits / n_windows;
+    const int cap_hits = (int)std::min<long long>(2048, std::max<long long>(512, (2 * mean + 63) & ~63LL));
+    hk::IterParams q{};
+    int ctas = 4;
+    for (; ctas >= 1; --ctas) {
+        const size_t share = std::min(ctx->smem_optin + 128 - fa.sharedSizeBytes,
+                                      ctx->smem_per_sm / (size_t)ctas - 1024 - fa.sharedSizeBytes);
+        const size_t fixed = hk::iter_smem_bytes(nb, cap_hits, 0);
+        if (fixed + 1536 * 4 <= share) {
+            q.cap_hits = cap_hits;
+            q.cap_list = (int)std::min<size_t>(8192, (share - fixed) / 4) & ~31;
+            break;
+        }
+    }
+    // the rest: 512 threads, tiles of 32 word rows beside the stage of hits and
+    // the kernel's static shared variables (small tiles let more of them be
     // skipped once their count bound falls; 64 or 128 word rows were slower)
-    hough_launch l{512, 32, HOUGH_ITER_MAX_HITS, 1};
-    const size_t stage = (size_t)HOUGH_ITER_MAX_HITS * 12;
-    cudaFuncAttributes fa{};
-    if (cudaFuncGetAttributes(&fa, hk::iterative_kernel) != cudaSuccess)
-        return fail(ctx, HOUGH_ERR_CUDA);
-    const size_t room = ctx->smem_optin + 128 > fa.sharedSizeBytes
-                            ? ctx->smem_optin + 128 - fa.sharedSizeBytes : 0;
-    // the find's narrowed tiles
-    const size_t smem = (size_t)l.word_rows * tile_bins(ctx, l.word_rows) * 4 + stage;
-    if (smem > room)
+    const size_t room = ctx->smem_optin + 128 > fb.sharedSizeBytes
+                            ? ctx->smem_optin + 128 - fb.sharedSizeBytes : 0;
+    const size_t smem_tiles = (size_t)32 * nb * 4 + (size_t)HOUGH_ITER_MAX_HITS * 12;
+    if (smem_tiles > room || ctas < 1)
         return fail(ctx, HOUGH_ERR_UNSUPPORTED_SHAPE);
-    if (raise_smem_limit(reinterpret_cast<const void *>(hk::iterative_kernel), smem) != HOUGH_OK)
+    const size_t smem = hk::iter_smem_bytes(nb, q.cap_hits, q.cap_list);
+    void (*kernel)(hk::IterParams) = ctas == 1 ? hk::iterative_kernel_512
+                                     : ctas == 2 ? hk::iterative_kernel_256
+                                                 : hk::iterative_kernel_128;
+    const int threads = ctas == 1 ? 512 : ctas == 2 ? 256 : 128;
+    if (raise_smem_limit(reinterpret_cast<const void *>(kernel), smem) != HOUGH_OK ||
+        raise_smem_limit(reinterpret_cast<const void *>(hk::iterative_tiles_kernel), smem_tiles) !=
+            HOUGH_OK)
         return fail(ctx, HOUGH_ERR_CUDA);
+    const hough_launch l{512, 32, HOUGH_ITER_MAX_HITS, 1};
     hough_tracks out{};
     out.hit_track = hit_track;
     out.window_status = window_status;
-    hk::IterParams q{};
     q.k = make_params(ctx, hits, window_offsets, n_windows, &out, nullptr, l);
     q.max_tracks = max_tracks;
     q.tracks = reinterpret_cast<int4 *>(tracks);
     q.n_tracks = n_tracks;
-    const long long grid = std::min<long long>(n_windows, (long long)ctx->num_sms);
-    hk::iterative_kernel<<<(unsigned)grid, 512, smem, (cudaStream_t)stream>>>(q);
+    q.work = counter_for(ctx, (cudaStream_t)stream);     // none while a capture cannot allocate it
+    const long long grid = std::min<long long>(n_windows, (long long)ctx->num_sms * ctas);
+    kernel<<<(unsigned)grid, threads, smem, (cudaStream_t)stream>>>(q);
     if (cudaGetLastError() != cudaSuccess)
         return fail(ctx, HOUGH_ERR_CUDA);
-    ctx->launches += 1;
+    const long long grid_tiles = std::min<long long>(n_windows, (long long)ctx->num_sms);
+    hk::iterative_tiles_kernel<<<(unsigned)grid_tiles, 512, smem_tiles, (cudaStream_t)stream>>>(q);
+    if (cudaGetLastError() != cudaSuccess)
+        return fail(ctx, HOUGH_ERR_CUDA);
+    ctx->launches += 2;
     return HOUGH_OK;
 }
 

@@ -4,12 +4,15 @@
 // order), stop below T, else give track k every remaining hit within tol
 // bins of it in its row, remove them and vote again.
 //
-// One CTA per window (grid-stride).  The window's valid hits are staged in
-// shared memory with their window-local indices; every iteration runs the
-// theta tiles of the find kernel's vote loop (its narrowed tiles of 32 word
-// rows, stored without guard columns) and a block maximum over each tile's
-// counters, then marks the line's hits and compacts them out of the stage in
-// order.
+// Two kernels.  iterative_kernel takes the windows it has room for: it votes
+// the window's hits once, tile by tile as the find does, and lists every bin
+// with at least T votes.  Counts only fall as tracks leave, so the highest bin
+// of every iteration is a listed one, and taking a track's hits back is a few
+// comparisons per listed bin: an iteration is two passes over short lists and
+// two barriers, and no accumulator is kept.  iterative_tiles_kernel takes the
+// rest: every iteration re-votes the find kernel's theta tiles (32 word rows,
+// stored without guard columns), leaving out those that cannot hold the
+// highest bin.
 #pragma once
 
 #include "hough_kernels.cuh"
@@ -21,7 +24,16 @@ struct IterParams {
     int max_tracks;
     int4 *tracks;               // [n_windows * max_tracks]: theta, rho, votes, n_hits
     int32_t *n_tracks;          // [n_windows]
+    int cap_hits, cap_list;     // iterative_kernel: staged hits and listed bins
+    unsigned *work;             // next-window and finished-CTA counters, as the find's (null: windows in turn)
 };
+
+constexpr int kIterLeft = -1;   // n_tracks of a window left to iterative_tiles_kernel
+
+__host__ __device__ inline size_t iter_smem_bytes(int n_b, int cap_hits, int cap_list)
+{
+    return tile_words(32, n_b) * 4 + (size_t)cap_hits * 18 + (size_t)cap_list * 4;
+}
 
 // Stage the window's valid hits (in order) with their window-local indices;
 // invalid hits get hit_track = -2, valid ones -1.  Returns the staged count
@@ -213,13 +225,14 @@ __device__ unsigned long long iter_best(const KParams &p, uint32_t *acc, const i
     return best;
 }
 
-__global__ void __launch_bounds__(512, 1) iterative_kernel(IterParams q)
+__global__ void __launch_bounds__(512, 1) iterative_tiles_kernel(IterParams q)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ WinScalars ws;
     __shared__ unsigned long long red[16];
     __shared__ int wtot[32];
     __shared__ int taken;
+    __shared__ unsigned todo[16];
     __shared__ int ub[HOUGH_MAX_THETA / 32];      // per-tile bounds (at most n_theta / 32 tiles)
     __shared__ unsigned done[HOUGH_MAX_THETA / 32 / 32];
     const KParams &p = q.k;
@@ -228,7 +241,210 @@ __global__ void __launch_bounds__(512, 1) iterative_kernel(IterParams q)
     int2 *stage = reinterpret_cast<int2 *>(smem + (size_t)p.word_rows * p.n_b * 4);
     int *sidx = reinterpret_cast<int *>(stage + p.hit_stage);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (long long w = blockIdx.x; w < p.n_windows; w += gridDim.x) {
+    // this CTA's windows, 512 looked at together: most are done already
+    for (long long k0 = 0; k0 * gridDim.x < p.n_windows; k0 += 512) {
+        const long long mine = (k0 + threadIdx.x) * gridDim.x + blockIdx.x;
+        const unsigned left = __ballot_sync(0xffffffffu, mine < p.n_windows && q.n_tracks[mine] == kIterLeft);
+        __syncthreads();
+        if (lane == 0)
+            todo[warp] = left;
+        __syncthreads();
+        for (int x = 0; x < 512; ++x) {
+            if (!(todo[x >> 5] >> (x & 31) & 1u)) {
+                x |= todo[x >> 5] ? 0 : 31;
+                continue;
+            }
+            const long long w = (k0 + x) * gridDim.x + blockIdx.x;
+            const long long beg = p.offsets[w], end = p.offsets[w + 1];
+            const int H = (int)(end - beg);
+            if (threadIdx.x == 0)
+                ws.flags = 0u;
+            __syncthreads();
+            int nv = iter_stage(p, beg, H, stage, sidx, wtot);
+            int found = 0;
+            unsigned flags = 0u;
+            if (nv < 0) {
+                flags |= HOUGH_WIN_TOO_LARGE;
+                nv = 0;
+            }
+            int width = 0;                               // counter fields per word of the bounds
+            while (found < q.max_tracks && nv > 0) {
+                const int P = nv <= 255 ? 4 : (nv <= 65535 ? 2 : 1);
+                if (P != width) {                        // new tiling: no bound known yet
+                    for (int i = threadIdx.x; i < HOUGH_MAX_THETA / 32; i += blockDim.x)
+                        ub[i] = 0x7fffffff;
+                    __syncthreads();
+                    width = P;
+                }
+                unsigned long long best;
+                if (P == 4)
+                    best = iter_best<4>(p, acc, stage, nv, red, ws, ub, done, T);
+                else if (P == 2)
+                    best = iter_best<2>(p, acc, stage, nv, red, ws, ub, done, T);
+                else
+                    best = iter_best<1>(p, acc, stage, nv, red, ws, ub, done, T);
+                const int votes = (int)(best >> 32);
+                if (votes < T)
+                    break;
+                const unsigned tb = 0xffffffffu - (unsigned)(best & 0xffffffffu);
+                const int bt = (int)(tb >> 16), bb = (int)(tb & 0xffffu);
+                const int c = __ldg(p.C + bt), s = __ldg(p.S + bt);
+                if (threadIdx.x == 0)
+                    taken = 0;
+                __syncthreads();
+                // mark the line's hits and compact the rest, in order, in place
+                int kept = 0, mine = 0;
+                for (int c0 = 0; c0 < nv; c0 += blockDim.x) {
+                    const int i = c0 + threadIdx.x;
+                    int2 h = make_int2(0, 0);
+                    int idx = 0;
+                    bool keep = false;
+                    if (i < nv) {
+                        h = stage[i];
+                        idx = sidx[i];
+                        const int d = rho_bin(h.x, h.y, c, s, p.D, p.K) - bb;
+                        if (d <= p.tol && d >= -p.tol) {
+                            p.hit_track[beg + idx] = found;
+                            ++mine;
+                        } else {
+                            keep = true;
+                        }
+                    }
+                    const unsigned m = __ballot_sync(0xffffffffu, keep);
+                    if (lane == 0)
+                        wtot[warp] = __popc(m);
+                    __syncthreads();
+                    int pre = 0, tot = 0;
+                    for (int k = 0; k < nw; ++k) {
+                        const int v = wtot[k];
+                        pre += k < warp ? v : 0;
+                        tot += v;
+                    }
+                    if (keep) {
+                        const int pos = kept + pre + __popc(m & lanemask_lt());
+                        stage[pos] = h;
+                        sidx[pos] = idx;
+                    }
+                    kept += tot;
+                    __syncthreads();
+                }
+    #pragma unroll
+                for (int d = 16; d > 0; d >>= 1)
+                    mine += __shfl_xor_sync(0xffffffffu, mine, d);
+                if (lane == 0 && mine)
+                    atomicAdd(&taken, mine);
+                __syncthreads();
+                if (threadIdx.x == 0)
+                    q.tracks[(size_t)w * q.max_tracks + found] = make_int4(bt, bb, votes, taken);
+                nv = kept;
+                ++found;
+                __syncthreads();
+        }
+        if (threadIdx.x == 0) {
+            q.n_tracks[w] = found;
+            p.status[w] = flags | ws.flags;
+        }
+        __syncthreads();
+        }
+    }
+}
+
+// iterative_kernel's scalars.
+struct IterScalars {
+    int n_list;          // bins listed (and refused places past the end)
+    int taken[2];        // hits of the last track, in turn
+    unsigned sum;        // votes in the counters of the tiles so far
+    unsigned int flags;
+};
+
+// Bins of a voted tile with at least `floor` votes, as keys: votes, then the
+// first bin in row-major order, larger is better.
+template <class S>
+__device__ __forceinline__ void iter_list(const KParams &p, unsigned acc0, int t0, int lo, int floor,
+                                          bool count, uint32_t *list, int cap, IterScalars &is)
+{
+    const int lane = threadIdx.x & 31;
+    const int n4 = p.n_b * 8;
+    const unsigned low = (1u << (p.tb + p.bb)) - 1u;
+    unsigned sum = 0u;
+    for (int x = threadIdx.x; x < n4; x += S::threads()) {
+        const uint4 v = lds128(acc0 + (unsigned)x * 16u);
+        if (count) {
+            sum = __dp4a(v.x, 0x01010101u, sum);
+            sum = __dp4a(v.y, 0x01010101u, sum);
+            sum = __dp4a(v.z, 0x01010101u, sum);
+            sum = __dp4a(v.w, 0x01010101u, sum);
+        }
+        if (!quad_has<4>(v, floor))
+            continue;
+        const uint32_t y[4] = {v.x, v.y, v.z, v.w};
+        const int b = (x >> 3) + lo, t = t0 + (x & 7) * 16;
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                const int n = field<4>(y[e], s);
+                if (n >= floor) {
+                    const int at = atomicAdd(&is.n_list, 1);
+                    if (at < cap)
+                        list[at] = (unsigned)n << (p.tb + p.bb) | (low - ((unsigned)(t + e * 4 + s) << p.bb | (unsigned)b));
+                }
+            }
+    }
+    if (count) {
+        sum = __reduce_add_sync(0xffffffffu, sum);
+        if (lane == 0)
+            atomicAdd(&is.sum, sum);
+    }
+}
+
+// One window per CTA (grid-stride): the staged valid hits, one 8-bit tile of
+// 128 rows, and the list of the bins with at least `floor` votes (T, or more
+// while the list cannot hold every bin >= T: its tracks are taken first, and
+// the hits left are voted again).  Left to iterative_tiles_kernel: windows of
+// more hits than are staged or than a key counts, of more than 255 hits where
+// the votes cannot be counted back from the bytes (or one overflowed), and
+// windows with more equal bins than the list holds.
+//
+// Bound: instructions -- the vote and scan of the find (once), then per track
+// about 5 per listed bin and hit of the track.  5000 windows, 512 x 512, by
+// re-voted tiles and by lists: 142 hits 4.53 -> 0.51 ms, 285 hits 9.3 -> 1.7 ms,
+// 570 hits 16.3 -> 3.0 ms.  (All rows' 8-bit counters kept in shared memory, the
+// votes taken back and the whole accumulator scanned per track: 2.0 ms at 142
+// hits, one CTA per SM and four barriers a track.)
+template <int NT>
+__device__ __forceinline__ void iter_body(const IterParams &q)
+{
+    using S = Shape<NT, 32>;
+    constexpr int nw = NT / 32;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ WinScalars ws;
+    __shared__ IterScalars is;
+    __shared__ int wtot[32];
+    __shared__ int hist[64];
+    const KParams &p = q.k;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = lanemask_lt();
+    const int NB = p.n_b, shift = p.tb + p.bb;
+    uint32_t *tile = reinterpret_cast<uint32_t *>(smem);
+    int2 *stage = reinterpret_cast<int2 *>(smem + tile_words(32, NB) * 4);
+    int2 *tk = stage + q.cap_hits;                       // hits of the last track
+    uint32_t *list = reinterpret_cast<uint32_t *>(tk + q.cap_hits);
+    uint16_t *sidx = reinterpret_cast<uint16_t *>(list + q.cap_list);
+    const unsigned acc0 = (unsigned)__cvta_generic_to_shared(tile) + kGuard * 128u;
+    const int n_tiles = (p.n_theta + 127) / 128;
+    const int32_t *lo_row = p.lo_tab ? p.lo_tab + 2 * p.lo_stride : nullptr;
+    zero_tile<S>(p, tile);
+    auto next = [&](long long w) {
+        if (!q.work)
+            return w + gridDim.x;
+        __syncthreads();
+        if (threadIdx.x == 0)
+            ws.next_w = (int)gridDim.x + (int)atomicAdd(q.work, 1u);
+        __syncthreads();
+        return (long long)ws.next_w;
+    };
+    for (long long w = blockIdx.x; w < p.n_windows; w = next(w)) {
         const long long beg = p.offsets[w], end = p.offsets[w + 1];
         if (!(beg >= 0 && beg <= end && end <= p.n_hits && end - beg < (1ll << 30))) {
             if (threadIdx.x == 0) {
@@ -238,95 +454,238 @@ __global__ void __launch_bounds__(512, 1) iterative_kernel(IterParams q)
             continue;
         }
         const int H = (int)(end - beg);
+        if (H > q.cap_hits || H >= 1 << (32 - shift) || (H > 255 && !(p.in_range && H <= 8 * NB))) {
+            if (threadIdx.x == 0)
+                q.n_tracks[w] = kIterLeft;
+            continue;
+        }
+        __syncthreads();                                 // the last window's reads are over
         if (threadIdx.x == 0)
             ws.flags = 0u;
-        __syncthreads();
-        int nv = iter_stage(p, beg, H, stage, sidx, wtot);
-        int found = 0;
-        unsigned flags = 0u;
-        if (nv < 0) {
-            flags |= HOUGH_WIN_TOO_LARGE;
-            nv = 0;
-        }
-        int width = 0;                               // counter fields per word of the bounds
-        while (found < q.max_tracks && nv > 0) {
-            const int P = nv <= 255 ? 4 : (nv <= 65535 ? 2 : 1);
-            if (P != width) {                        // new tiling: no bound known yet
-                for (int i = threadIdx.x; i < HOUGH_MAX_THETA / 32; i += blockDim.x)
-                    ub[i] = 0x7fffffff;
-                __syncthreads();
-                width = P;
+        // stage the valid hits with their window-local indices
+        int nv = 0;
+        for (int c0 = 0; c0 < H; c0 += NT) {
+            const int i = c0 + threadIdx.x;
+            int phi = 0, z = 0;
+            bool ok = false;
+            if (i < H) {
+                ok = load_hit(p, beg + i, phi, z);
+                p.hit_track[beg + i] = ok ? -1 : -2;
             }
-            unsigned long long best;
-            if (P == 4)
-                best = iter_best<4>(p, acc, stage, nv, red, ws, ub, done, T);
-            else if (P == 2)
-                best = iter_best<2>(p, acc, stage, nv, red, ws, ub, done, T);
-            else
-                best = iter_best<1>(p, acc, stage, nv, red, ws, ub, done, T);
-            const int votes = (int)(best >> 32);
-            if (votes < T)
-                break;
-            const unsigned tb = 0xffffffffu - (unsigned)(best & 0xffffffffu);
-            const int bt = (int)(tb >> 16), bb = (int)(tb & 0xffffu);
-            const int c = __ldg(p.C + bt), s = __ldg(p.S + bt);
-            if (threadIdx.x == 0)
-                taken = 0;
+            const unsigned m = __ballot_sync(0xffffffffu, ok);
+            if (lane == 0)
+                wtot[warp] = __popc(m);
             __syncthreads();
-            // mark the line's hits and compact the rest, in order, in place
-            int kept = 0, mine = 0;
-            for (int c0 = 0; c0 < nv; c0 += blockDim.x) {
-                const int i = c0 + threadIdx.x;
-                int2 h = make_int2(0, 0);
-                int idx = 0;
-                bool keep = false;
-                if (i < nv) {
-                    h = stage[i];
-                    idx = sidx[i];
-                    const int d = rho_bin(h.x, h.y, c, s, p.D, p.K) - bb;
-                    if (d <= p.tol && d >= -p.tol) {
-                        p.hit_track[beg + idx] = found;
-                        ++mine;
-                    } else {
-                        keep = true;
+            const int c = lane < nw ? wtot[lane] : 0;
+            const int pos = nv + (int)__reduce_add_sync(0xffffffffu, (unsigned)(lane < warp ? c : 0)) + __popc(m & lt);
+            if (ok) {
+                stage[pos] = make_int2(phi, z);
+                sidx[pos] = (uint16_t)i;
+            }
+            nv += (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
+            __syncthreads();
+        }
+        int found = 0;
+        bool left = false;
+        while (nv > 0 && found < q.max_tracks) {
+            // vote every tile and list its bins >= floor
+            int floor = p.T;
+            if (threadIdx.x == 0) {
+                is.n_list = 0;
+                is.sum = 0u;
+                is.taken[0] = is.taken[1] = 0;
+            }
+            __syncthreads();
+            for (int k = 0; k < n_tiles && !left; ++k) {
+                const int t0 = k * 128;
+                const int lo = lo_row ? __ldg(lo_row + k) : 0;
+                if (p.in_range && t0 + 128 <= p.n_theta)
+                    vote_tile<S, 4, true>(p, acc0, 0u, stage, nv, t0, lo, ws);
+                else
+                    vote_tile<S, 4, false>(p, acc0, 0u, stage, nv, t0, lo, ws);
+                int before = is.n_list;                  // of the tiles before (no one adds to it now)
+                __syncthreads();
+                iter_list<S>(p, acc0, t0, lo, floor, nv > 255, list, q.cap_list, is);
+                __syncthreads();
+                while (is.n_list > q.cap_list) {
+                    // raise the floor until half the list is free, drop what
+                    // falls below it, and list the tile again
+                    for (int i = threadIdx.x; i < 64; i += NT)
+                        hist[i] = 0;
+                    __syncthreads();
+                    for (int i = threadIdx.x; i < q.cap_list; i += NT)
+                        atomicAdd(&hist[min((int)(list[i] >> shift), 63)], 1);
+                    __syncthreads();
+                    int n = 0, v = 64;
+                    while (v > 0 && n + hist[v - 1] <= q.cap_list / 2)
+                        n += hist[--v];
+                    floor = max(floor + 1, v);
+                    left = left || v > 63;               // too many to tell apart
+                    __syncthreads();
+                    if (warp == 0) {
+                        int m = 0;
+                        for (int i0 = 0; i0 < before; i0 += 32) {
+                            const uint32_t key = i0 + lane < before ? list[i0 + lane] : 0u;
+                            const unsigned mk = __ballot_sync(0xffffffffu, (int)(key >> shift) >= floor);
+                            if (mk >> lane & 1u)
+                                list[m + __popc(mk & lt)] = key;
+                            m += __popc(mk);
+                            __syncwarp();
+                        }
+                        if (lane == 0)
+                            is.n_list = m;
+                    }
+                    __syncthreads();
+                    before = is.n_list;
+                    __syncthreads();
+                    iter_list<S>(p, acc0, t0, lo, floor, false, list, q.cap_list, is);
+                    __syncthreads();
+                    if (left)
+                        break;
+                }
+                zero_tile<S>(p, tile);
+                __syncthreads();
+            }
+            if (nv > 255 && is.sum != (unsigned)nv * (unsigned)p.n_theta)
+                left = true;                             // a byte overflowed
+            if (left)
+                break;
+            // this thread's hits still unassigned: bit k for hit k NT + threadIdx.x
+            unsigned alive = 0u;
+            for (int k = 0; k * NT + (int)threadIdx.x < nv; ++k)
+                alive |= 1u << k;
+            // each warp keeps its share of the list, in place, and drops the
+            // bins that fall below the floor
+            const int first = found, share = (is.n_list + nw - 1) / nw;
+            uint32_t *mine = list + warp * share;
+            int n = max(min(share, is.n_list - warp * share), 0);
+            int n_tk = 0;
+            for (;;) {
+                // take the last track's votes from the listed bins; the best left
+                uint32_t best = 0u;
+                int kept = 0;
+                for (int i0 = 0; i0 < n; i0 += 32) {
+                    uint32_t key = i0 + lane < n ? mine[i0 + lane] : 0u;
+                    if (n_tk > 0) {
+                        // a hit is in the bin when its sum is within 2^K of the bin's
+                        // first (mod 2^32: the sums span less than 2^32 - 2^K)
+                        const unsigned at = ((1u << shift) - 1u) - (key & ((1u << shift) - 1u));
+                        const int t = min((int)(at >> p.bb), p.n_theta - 1);
+                        const unsigned c = (unsigned)__ldg(p.C + t), s = (unsigned)__ldg(p.S + t);
+                        const unsigned d = (unsigned)p.D - ((at & ((1u << p.bb) - 1u)) << p.K);
+                        const unsigned one = 1u << p.K;
+                        const int4 *pair = reinterpret_cast<const int4 *>(tk);
+                        unsigned off = 0u;
+#pragma unroll 4
+                        for (int x = 0; x < n_tk >> 1; ++x) {
+                            const int4 h = pair[x];
+                            off += (unsigned)h.x * c + (unsigned)h.y * s + d < one ? 1u : 0u;
+                            off += (unsigned)h.z * c + (unsigned)h.w * s + d < one ? 1u : 0u;
+                        }
+                        if (n_tk & 1) {
+                            const int2 h = tk[n_tk - 1];
+                            off += (unsigned)h.x * c + (unsigned)h.y * s + d < one ? 1u : 0u;
+                        }
+                        key -= off << shift;
+                    }
+                    const bool ok = i0 + lane < n && (int)(key >> shift) >= floor;
+                    const unsigned mk = __ballot_sync(0xffffffffu, ok);
+                    if (ok)
+                        mine[kept + __popc(mk & lt)] = key;
+                    kept += __popc(mk);
+                    best = max(best, ok ? key : 0u);
+                    __syncwarp();
+                }
+                n = kept;
+                best = __reduce_max_sync(0xffffffffu, best);
+                if (lane == 0)
+                    wtot[warp] = (int)best;
+                __syncthreads();
+                best = __reduce_max_sync(0xffffffffu, lane < nw ? (unsigned)wtot[lane] : 0u);
+                const int votes = (int)(best >> shift);
+                if (best == 0u || votes < floor || found == q.max_tracks)
+                    break;
+                const unsigned at = ((1u << shift) - 1u) - (best & ((1u << shift) - 1u));
+                const int bt = (int)(at >> p.bb), bb = (int)(at & ((1u << p.bb) - 1u));
+                const int c = __ldg(p.C + bt), s = __ldg(p.S + bt);
+                int &taken = is.taken[found & 1];
+                for (int k = 0; k * NT < nv; ++k) {
+                    const int i = k * NT + (int)threadIdx.x;
+                    bool take = false;
+                    int2 h = make_int2(0, 0);
+                    if (alive >> k & 1u) {
+                        h = stage[i];
+                        const int d = rho_bin(h.x, h.y, c, s, p.D, p.K) - bb;
+                        take = d <= p.tol && d >= -p.tol;
+                    }
+                    const unsigned m = __ballot_sync(0xffffffffu, take);
+                    if (m != 0u) {
+                        int base = 0;
+                        if (lane == 0)
+                            base = atomicAdd(&taken, __popc(m));
+                        base = __shfl_sync(0xffffffffu, base, 0);
+                        if (take) {
+                            alive &= ~(1u << k);
+                            tk[base + __popc(m & lt)] = h;
+                            p.hit_track[beg + sidx[i]] = found;
+                        }
                     }
                 }
+                __syncthreads();
+                n_tk = taken;
+                if (threadIdx.x == 0) {
+                    q.tracks[(size_t)w * q.max_tracks + found] = make_int4(bt, bb, votes, n_tk);
+                    is.taken[(found + 1) & 1] = 0;
+                }
+                ++found;
+            }
+            if (floor == p.T || found == q.max_tracks)
+                break;
+            if (found == first) {
+                left = true;                             // more equal bins than the list holds
+                break;
+            }
+            // the hits left, in order, for the next list
+            int kept = 0;
+            __syncthreads();
+            for (int k = 0; k * NT < nv; ++k) {
+                const int i = k * NT + (int)threadIdx.x;
+                const bool keep = alive >> k & 1u;
+                const int2 h = keep ? stage[i] : make_int2(0, 0);
+                const uint16_t ix = keep ? sidx[i] : (uint16_t)0;
                 const unsigned m = __ballot_sync(0xffffffffu, keep);
                 if (lane == 0)
                     wtot[warp] = __popc(m);
                 __syncthreads();
-                int pre = 0, tot = 0;
-                for (int k = 0; k < nw; ++k) {
-                    const int v = wtot[k];
-                    pre += k < warp ? v : 0;
-                    tot += v;
-                }
+                const int c = lane < nw ? wtot[lane] : 0;
+                const int pos = kept + (int)__reduce_add_sync(0xffffffffu, (unsigned)(lane < warp ? c : 0)) + __popc(m & lt);
                 if (keep) {
-                    const int pos = kept + pre + __popc(m & lanemask_lt());
                     stage[pos] = h;
-                    sidx[pos] = idx;
+                    sidx[pos] = ix;
                 }
-                kept += tot;
+                kept += (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
                 __syncthreads();
             }
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1)
-                mine += __shfl_xor_sync(0xffffffffu, mine, d);
-            if (lane == 0 && mine)
-                atomicAdd(&taken, mine);
-            __syncthreads();
-            if (threadIdx.x == 0)
-                q.tracks[(size_t)w * q.max_tracks + found] = make_int4(bt, bb, votes, taken);
             nv = kept;
-            ++found;
-            __syncthreads();
         }
         if (threadIdx.x == 0) {
-            q.n_tracks[w] = found;
-            p.status[w] = flags | ws.flags;
+            q.n_tracks[w] = left ? kIterLeft : found;
+            p.status[w] = ws.flags;
         }
-        __syncthreads();
+    }
+    // the last CTA to finish resets the counters for the next launch
+    if (q.work && threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(q.work + 1, 1u) == gridDim.x - 1) {
+            atomicExch(q.work, 0u);
+            atomicExch(q.work + 1, 0u);
+            __threadfence();
+        }
     }
 }
+
+__global__ void __launch_bounds__(128, 4) iterative_kernel_128(IterParams q) { iter_body<128>(q); }
+__global__ void __launch_bounds__(256, 2) iterative_kernel_256(IterParams q) { iter_body<256>(q); }
+__global__ void __launch_bounds__(512, 1) iterative_kernel_512(IterParams q) { iter_body<512>(q); }
 
 }  // namespace hk
