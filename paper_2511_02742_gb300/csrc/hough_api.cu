@@ -353,6 +353,22 @@ bool hits_ok(const hough_hits *h)
     return true;
 }
 
+// The detector box of the kernels: 0 <= phi < 360 deg, z_min <= z <= z_end,
+// its ends cut to what 32-bit coordinates can reach.
+hk::HitBox hit_box(const hough_geometry &g, bool raw)
+{
+    hk::HitBox b{};
+    const long long phi_end = 360LL * g.phi_u_per_deg;
+    b.raw = raw ? 1 : 0;
+    b.vane_step = (int)(phi_end / g.n_vanes);
+    b.z_min = g.z_min_u;
+    b.z_pitch = g.z_pitch_u;
+    b.z_half = g.z_pitch_u / 2;
+    b.z_end = (int)std::min<long long>((long long)g.z_min_u + (long long)g.n_z_strips * g.z_pitch_u, INT_MAX);
+    b.phi_end = (unsigned)std::min<long long>(phi_end, 1LL << 31);
+    return b;
+}
+
 // narrow: the find kernel's narrowed tiles (the other kernels that take these
 // parameters keep full-width tiles)
 hk::KParams make_params(const hough_ctx *ctx, const hough_hits *hits, const int64_t *offsets,
@@ -365,13 +381,7 @@ hk::KParams make_params(const hough_ctx *ctx, const hough_hits *hits, const int6
     p.a = raw ? hits->vane : hits->phi_q;
     p.b = raw ? hits->strip : hits->z_q;
     p.n_hits = hits->n_hits;
-    p.raw = raw ? 1 : 0;
-    p.vane_step = (int)(360LL * g.phi_u_per_deg / g.n_vanes);
-    p.z_min_u = g.z_min_u;
-    p.z_pitch_u = g.z_pitch_u;
-    p.z_half = g.z_pitch_u / 2;
-    p.phi_end = 360LL * g.phi_u_per_deg;
-    p.z_end = (long long)g.z_min_u + (long long)g.n_z_strips * g.z_pitch_u;
+    p.box = hit_box(g, raw);
     p.offsets = reinterpret_cast<const long long *>(offsets);
     p.n_windows = n_windows;
     p.C = ctx->d_C;
@@ -891,6 +901,10 @@ int hough_find_coarse_fine(hough_ctx *ctx, const hough_hits *hits, const int64_t
             cudaFree(d);
             return fail(ctx, HOUGH_ERR_CUDA);
         }
+        ctx->cf_in_range = box_votes_in_range(&ctx->g, hk::kCfCoarseT, hk::kCfCoarseR, tab.data(),
+                                              tab.data() + hk::kCfCoarseT, ctx->cf_D[0],
+                                              ctx->cf_K[0]);
+        std::memcpy(ctx->cf_coarse, tab.data(), sizeof ctx->cf_coarse);
         ctx->d_cf = d;
     }
     const hough_geometry &g = ctx->g;
@@ -899,23 +913,18 @@ int hough_find_coarse_fine(hough_ctx *ctx, const hough_hits *hits, const int64_t
     p.a = raw ? hits->vane : hits->phi_q;
     p.b = raw ? hits->strip : hits->z_q;
     p.n_hits = hits->n_hits;
-    p.raw = raw ? 1 : 0;
-    p.vane_step = (int)(360LL * g.phi_u_per_deg / g.n_vanes);
-    p.z_min_u = g.z_min_u;
-    p.z_pitch_u = g.z_pitch_u;
-    p.z_half = g.z_pitch_u / 2;
-    p.phi_end = 360LL * g.phi_u_per_deg;
-    p.z_end = (long long)g.z_min_u + (long long)g.n_z_strips * g.z_pitch_u;
+    p.box = hit_box(g, raw);
     p.offsets = reinterpret_cast<const long long *>(window_offsets);
     p.n_windows = n_windows;
-    p.Cc = ctx->d_cf;
-    p.Sc = ctx->d_cf + hk::kCfCoarseT;
+    std::memcpy(p.Cc, ctx->cf_coarse, sizeof p.Cc);
+    std::memcpy(p.Sc, ctx->cf_coarse + hk::kCfCoarseT, sizeof p.Sc);
     p.Cf = ctx->d_cf + 2 * hk::kCfCoarseT;
     p.Sf = ctx->d_cf + 2 * hk::kCfCoarseT + hk::kCfFineT;
     p.Dc = (int)ctx->cf_D[0];
     p.Kc = ctx->cf_K[0];
     p.Df = (int)ctx->cf_D[1];
     p.Kf = ctx->cf_K[1];
+    p.in_range = ctx->cf_in_range ? 1 : 0;
     p.T = ctx->th.vote_threshold;
     p.tol = ctx->th.assoc_tol_bins;
     p.lines = lines;

@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(32) extend_kernel(ExtParams q)
     int32_t *bstart = reinterpret_cast<int32_t *>(bucket + cap);   // cap is a multiple of 8
     int32_t *bcur = bstart + nv + 1;
     int16_t *line = reinterpret_cast<int16_t *>(bcur + nv);
-    const int vstep = p.vane_step;
+    const int vstep = p.box.vane_step;
 
     for (long long w = blockIdx.x; w < p.n_windows; w += gridDim.x) {
         const long long beg = p.offsets[w], end = p.offsets[w + 1];
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(32) extend_kernel(ExtParams q)
             const int ht = p.hit_track[beg + i];
             int v = -1;
             if (ok && ht != -2) {
-                if (p.raw)
+                if (p.box.raw)
                     v = __ldg(p.a + beg + i);
                 else if (phi % vstep == 0)
                     v = phi / vstep;

@@ -44,6 +44,8 @@ struct hough_ctx {
     // coarse (18 x 100) and fine (180 x 1000) tables of the two-stage search:
     // C then S of each, on the device; built on first use
     int32_t *d_cf = nullptr;
+    bool cf_in_range = false;
+    int32_t cf_coarse[36] = {};   // the coarse ones on the host (kernel arguments)
     // hough_accumulate's launch (threads per CTA, resident CTAs per SM),
     // worked out on its first call
     int acc_threads = 0, acc_occ = 0;

@@ -93,23 +93,6 @@ __device__ __forceinline__ unsigned long long block_max_u64(unsigned long long k
     return m;
 }
 
-// Whether some P-bit field of w equals v (v < 2^(32/P)): the fields of
-// y = w ^ (v in every field) that are zero, by the exact zero-field test
-// (y - 0x..01..01) & ~y & 0x..80..80 (non-zero iff some field of y is zero).
-template <int P>
-__device__ __forceinline__ bool has_field(uint32_t w, unsigned v)
-{
-    if constexpr (P == 1) {
-        return w == v;
-    } else if constexpr (P == 2) {
-        const uint32_t y = w ^ (v * 0x00010001u);
-        return ((y - 0x00010001u) & ~y & 0x80008000u) != 0u;
-    } else {
-        const uint32_t y = w ^ (v * 0x01010101u);
-        return ((y - 0x01010101u) & ~y & 0x80808080u) != 0u;
-    }
-}
-
 // The tile's highest bin as the key (count << 32) | (2^32 - 1 - (t << 16 | b)):
 // the highest count, then the first bin in row-major order.  Two passes over
 // the counters: the highest count (fields only: rows past n_theta never get a

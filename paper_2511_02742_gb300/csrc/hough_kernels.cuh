@@ -55,16 +55,21 @@ constexpr int kGuard = 3;       // zero columns around the stored bins of a row 
 constexpr int kHistBins = 64;   // peak-vote histogram; last bin = ">= 63"
 constexpr int kListCap = 160;   // flagged quads a warp holds: four steps' 128 and 31 left over
 
+// The detector box, and the units of strip addresses.
+struct HitBox {
+    int raw;                // strip addresses (vane, strip), else encoded (phi, z)
+    int vane_step;          // phi units per vane
+    int z_min, z_pitch, z_half;
+    int z_end;              // z_min + n_z_strips * pitch (at most INT_MAX)
+    unsigned phi_end;       // 360 deg in phi units (at most 2^31)
+};
+
 struct KParams {
     // hits
     const int32_t *a;   // phi_q, or vane when raw
     const int32_t *b;   // z_q, or strip when raw
     long long n_hits;
-    int raw;
-    int vane_step;      // phi units per vane
-    int z_min_u, z_pitch_u, z_half;
-    long long phi_end;  // 360 deg in phi units
-    long long z_end;    // z_min + n_z_strips * pitch
+    HitBox box;
     // windows
     const long long *offsets;
     long long n_windows;
@@ -180,19 +185,23 @@ __device__ __forceinline__ unsigned lanemask_lt()
     return m;
 }
 
-// Encoded (phi, z) of hit i, and whether it lies inside the detector box.
+// Encoded (phi, z) of a hit, and whether it lies inside the detector box: all
+// in 32 bits (a strip address whose phi or z does not fit wraps, as the
+// encoded arrays of hough_encode do).
+__device__ __forceinline__ bool encode_hit(const HitBox &box, int a, int b, int &phi, int &z)
+{
+    phi = a;
+    z = b;
+    if (box.raw) {
+        phi = (int)((unsigned)box.vane_step * (unsigned)a);
+        z = (int)((unsigned)box.z_min + (unsigned)box.z_pitch * (unsigned)b + (unsigned)box.z_half);
+    }
+    return (unsigned)phi < box.phi_end && z >= box.z_min && z <= box.z_end;
+}
+
 __device__ __forceinline__ bool load_hit(const KParams &p, long long i, int &phi, int &z)
 {
-    int a = __ldg(p.a + i);
-    int b = __ldg(p.b + i);
-    if (p.raw) {
-        phi = (int)((long long)p.vane_step * (long long)a);
-        z = (int)((long long)p.z_min_u + (long long)p.z_pitch_u * (long long)b + p.z_half);
-    } else {
-        phi = a;
-        z = b;
-    }
-    return phi >= 0 && (long long)phi < p.phi_end && z >= p.z_min_u && (long long)z <= p.z_end;
+    return encode_hit(p.box, __ldg(p.a + i), __ldg(p.b + i), phi, z);
 }
 
 // floor((phi*c + z*s + D) / 2^K): the tables' scale keeps the exact sum of
@@ -397,6 +406,23 @@ __device__ __forceinline__ bool quad_has(const uint4 &q, int T)
         constexpr uint32_t hi = P == 4 ? 0x80808080u : 0x80008000u;
         const uint32_t add = (uint32_t)max((P == 4 ? 128 : 32768) - T, 0) * one;
         return (((q.x + add) | q.x | (q.y + add) | q.y | (q.z + add) | q.z | (q.w + add) | q.w) & hi) != 0u;
+    }
+}
+
+// Whether some field of w equals v (v < 2^(32/P)): the fields of
+// y = w ^ (v in every field) that are zero, by the exact zero-field test
+// (y - 0x..01..01) & ~y & 0x..80..80 (non-zero iff some field of y is zero).
+template <int P>
+__device__ __forceinline__ bool has_field(uint32_t w, unsigned v)
+{
+    if constexpr (P == 1) {
+        return w == v;
+    } else if constexpr (P == 2) {
+        const uint32_t y = w ^ (v * 0x00010001u);
+        return ((y - 0x00010001u) & ~y & 0x80008000u) != 0u;
+    } else {
+        const uint32_t y = w ^ (v * 0x01010101u);
+        return ((y - 0x01010101u) & ~y & 0x80808080u) != 0u;
     }
 }
 
