@@ -211,7 +211,8 @@ int hough_tables(const hough_geometry *g, int n_theta, int n_rho, int32_t *C, in
  * array of 3 T entries, T = ceil(n_theta / 32); entries past a width's last
  * tile are 0) receives tile i's first bin for counter width 2^k.  Contexts
  * use these for the fixed-point find (not for HOUGH_FLAG_FP64 or
- * hough_find_noalloc, whose tiles store every bin).
+ * hough_find_noalloc, whose tiles store every bin; with HOUGH_FLAG_EXPORT_ACC
+ * *nb is rounded up to whole blocks of 32 bins and lo down to 8).
  * Errors: INVALID_ARG (null pointer, bad geometry or word_rows),
  * UNSUPPORTED_SHAPE (as hough_create).
  */

@@ -72,9 +72,11 @@ static bool box_votes_in_range(const hough_geometry *g, int n_theta, int n_rho, 
 // stored bins.  When a bin below 0 is reachable, lo is 0.
 // nb[WR index]; lo_all: [WR index][log2 P][tile], tiles ceil(n_theta / 32)
 // apart.
+// bin_align, lo_align: other multiples for NB (where it stays below n_rho) and
+// for lo (a power of two that divides n_rho and bin_align).
 static void narrow_tiles(const hough_geometry *g, int nt, int nr, const int32_t *C,
                          const int32_t *S, long long D, int K, int nb_out[3],
-                         std::vector<int32_t> &lo_all)
+                         std::vector<int32_t> &lo_all, int bin_align = 4, int lo_align = 4)
 {
     std::vector<long long> rlo(nt), rhi(nt);
     for (int t = 0; t < nt; ++t)
@@ -99,12 +101,13 @@ static void narrow_tiles(const hough_geometry *g, int nt, int nr, const int32_t 
                     nb = std::max(nb, b - a + 1);
             }
         }
-        nb = std::min<long long>((nb + 3 + 3) & ~3LL, nr);
+        nb = (nb + lo_align - 1 + bin_align - 1) / bin_align * bin_align;
+        nb = std::min<long long>(nb, nr);
         nb_out[wi] = (int)nb;
         for (int lp = 0; lp < 3; ++lp)
             for (int k = 0; k * (WR << lp) < nt; ++k)
                 lo_all[(size_t)(wi * 3 + lp) * stride + k] = (int32_t)(std::min(
-                    std::max(tlo[(size_t)lp * stride + k], 0LL), (long long)nr - nb) & ~3LL);
+                    std::max(tlo[(size_t)lp * stride + k], 0LL), (long long)nr - nb) & ~(long long)(lo_align - 1));
     }
 }
 
@@ -648,9 +651,24 @@ int hough_create(const hough_geometry *g, int n_theta, int n_rho, const hough_th
         // narrowed tiles (the FP64 variant's bins come from another formula,
         // so its tiles keep every bin)
         std::vector<int32_t> lo_all;
+        // with the export on, tiles of whole blocks of 32 bins that start on a
+        // 32-byte sector of the output
+        const bool exported = (th->flags & HOUGH_FLAG_EXPORT_ACC) != 0;
         narrow_tiles(&ctx->g, ctx->n_theta, ctx->n_rho, ctx->C.data(), ctx->S.data(), ctx->D,
-                     ctx->K, ctx->tile_nb, lo_all);
+                     ctx->K, ctx->tile_nb, lo_all, exported ? 32 : 4,
+                     exported && ctx->n_rho % 8 == 0 ? 8 : 4);
         ctx->lo_stride = (ctx->n_theta + 31) / 32;
+        // hough_accumulate's: blocks of 32 bins, whole 128-byte lines of the
+        // output where its rows are; full-width tiles where three CTAs per SM
+        // hold them (their stores are then whole rows: 2000 windows of 142 hits
+        // at 512 x 512, 349 us narrowed, 343 us full-width)
+        std::vector<int32_t> lo_acc((size_t)3 * ctx->lo_stride, 0);
+        int nb_acc[3] = {ctx->n_rho, 0, 0};
+        if (3 * (hk::tile_words(32, ctx->n_rho) * 4 + (size_t)hk::kAccStage * 8 + 2048) > ctx->smem_per_sm)
+            narrow_tiles(&ctx->g, ctx->n_theta, ctx->n_rho, ctx->C.data(), ctx->S.data(), ctx->D,
+                         ctx->K, nb_acc, lo_acc, 32, ctx->n_rho % 32 == 0 ? 32 : 4);
+        ctx->acc_nb = nb_acc[0];
+        lo_all.insert(lo_all.end(), lo_acc.begin(), lo_acc.begin() + 3 * ctx->lo_stride);
         if (cudaMalloc(&ctx->d_lo, sizeof(int32_t) * lo_all.size()) != cudaSuccess) {
             hough_destroy(ctx);
             return HOUGH_ERR_ALLOC;
@@ -952,32 +970,26 @@ int hough_accumulate(hough_ctx *ctx, const hough_hits *hits, const int64_t *wind
         return fail(ctx, HOUGH_ERR_INVALID_ARG);
     if (n_windows == 0)
         return HOUGH_OK;
-    // tiles of 32 word rows and a stage of 2048 hits; 512-thread CTAs where
-    // two or more fit on an SM, else one CTA of 1024 threads
-    const int word_rows = 32, hit_stage = 2048;
-    const size_t smem = hk::align_up((size_t)word_rows * ctx->n_rho * 4, 16) + (size_t)hit_stage * 8;
+    using Kernel = void (*)(hk::AccParams);
+    static const Kernel kernels[3] = {hk::accumulate_kernel_256, hk::accumulate_kernel_512,
+                                      hk::accumulate_kernel_1024};
+    const int hit_stage = hk::kAccStage;
+    const size_t smem = hk::tile_words(32, ctx->acc_nb) * 4 + (size_t)hit_stage * 8;
     if (ctx->acc_threads == 0) {
-        // worked out once per context
-        cudaFuncAttributes fa{};
-        if (cudaFuncGetAttributes(&fa, hk::accumulate_kernel) != cudaSuccess)
-            return fail(ctx, HOUGH_ERR_CUDA);
-        if (smem + fa.sharedSizeBytes > ctx->smem_optin)
-            return fail(ctx, HOUGH_ERR_UNSUPPORTED_SHAPE);
-        if (raise_smem_limit(reinterpret_cast<const void *>(hk::accumulate_kernel), smem) !=
-            HOUGH_OK)
-            return fail(ctx, HOUGH_ERR_CUDA);
-        int threads = 512, occ = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, hk::accumulate_kernel, threads,
-                                                          smem) != cudaSuccess)
-            return fail(ctx, HOUGH_ERR_CUDA);
-        if (occ < 2) {
-            threads = 1024;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, hk::accumulate_kernel,
-                                                              threads, smem) != cudaSuccess)
+        // worked out once per context: the most CTAs per SM that fit, of 256
+        // threads from three up, 512 for two and 1024 for one
+        int threads = 0, occ = 0;
+        for (int k = 0; k < 3; ++k) {
+            threads = 256 << k;
+            if (raise_smem_limit(reinterpret_cast<const void *>(kernels[k]), smem) != HOUGH_OK ||
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernels[k], threads, smem) !=
+                    cudaSuccess)
                 return fail(ctx, HOUGH_ERR_CUDA);
-            if (occ < 1)
-                return fail(ctx, HOUGH_ERR_UNSUPPORTED_SHAPE);
+            if (occ >= (k == 0 ? 3 : k == 1 ? 2 : 1))
+                break;
         }
+        if (occ < 1)
+            return fail(ctx, HOUGH_ERR_UNSUPPORTED_SHAPE);
         ctx->acc_threads = threads;
         ctx->acc_occ = occ;
     }
@@ -985,10 +997,23 @@ int hough_accumulate(hough_ctx *ctx, const hough_hits *hits, const int64_t *wind
     hough_tracks out{};
     out.acc = acc;
     out.window_status = window_status;
-    hough_launch l{threads, word_rows, hit_stage, occ};
-    const hk::KParams p = make_params(ctx, hits, window_offsets, n_windows, &out, nullptr, l, false);
-    const long long grid = std::min<long long>(n_windows, (long long)ctx->num_sms * occ);
-    hk::accumulate_kernel<<<(unsigned)grid, threads, smem, (cudaStream_t)stream>>>(p);
+    const hough_launch l{threads, 32, hit_stage, occ};
+    hk::AccParams q{};
+    q.k = make_params(ctx, hits, window_offsets, n_windows, &out, nullptr, l);
+    q.k.n_b = ctx->acc_nb;
+    q.k.lo_tab = ctx->d_lo + (size_t)9 * ctx->lo_stride;
+    // parts of whole 128-row tiles, about six per resident CTA (each part
+    // stages the window's hits again); whole windows where votes may miss the
+    // range (a window's status has one writer)
+    const int n_tiles = (ctx->n_theta + 127) / 128;
+    const long long ctas = (long long)ctx->num_sms * occ;
+    q.part_tiles = ctx->in_range
+                       ? (int)std::min<long long>(n_tiles, std::max<long long>(1, n_windows * n_tiles / (6 * ctas)))
+                       : n_tiles;
+    q.parts = (n_tiles + q.part_tiles - 1) / q.part_tiles;
+    const long long grid = std::min<long long>(n_windows * q.parts, ctas);
+    kernels[threads == 256 ? 0 : threads == 512 ? 1 : 2]
+        <<<(unsigned)grid, threads, smem, (cudaStream_t)stream>>>(q);
     if (cudaGetLastError() != cudaSuccess)
         return fail(ctx, HOUGH_ERR_CUDA);
     ctx->launches += 1;

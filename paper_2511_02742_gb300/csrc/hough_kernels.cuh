@@ -968,9 +968,10 @@ __device__ __forceinline__ int4 fields4(const uint4 &v, int s)
 // aligned.  Stored bins past the last whole block, tiles with rows past
 // n_theta and accumulators that are not 16-byte aligned go out with 4-byte
 // stores; the bins the tile does not store are written as zeros.
-template <class S, int P>
-__device__ void export_tile_end(const KParams &p, uint32_t *acc, int t0, int R, int lo,
-                                long long w)
+// SUM: returns this lane's share of the sum of the tile's bytes (P = 4).
+template <class S, int P, bool SUM = false>
+__device__ __forceinline__ unsigned export_tile_end(const KParams &p, uint32_t *acc, int t0, int R,
+                                                    int lo, long long w)
 {
     constexpr int CW = 32 / P;
     constexpr unsigned MASK = P == 1 ? 0xffffffffu : ((1u << CW) - 1u);
@@ -980,6 +981,7 @@ __device__ void export_tile_end(const KParams &p, uint32_t *acc, int t0, int R, 
     int32_t *out = p.acc + (size_t)w * p.n_theta * p.n_rho;
     const bool vec = (reinterpret_cast<uintptr_t>(p.acc) & 15u) == 0u;
     const bool fast = t0 + R <= p.n_theta && vec;
+    unsigned sum = 0u;
     for (int item = warp; item < G * nblk; item += nw) {
         const int g = item / nblk, j0 = (item - g * nblk) * 32;
         uint32_t *blk = acc + (size_t)(g * (NB + kGuard) + j0) * 32;
@@ -987,6 +989,10 @@ __device__ void export_tile_end(const KParams &p, uint32_t *acc, int t0, int R, 
 #pragma unroll
         for (int j = 0; j < 32; ++j)
             r[j] = blk[j * 32 + lane];                 // word (g*32 + lane, j0 + j)
+        if (SUM)
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+                sum = __dp4a(r[j], 0x01010101u, sum);
         __syncwarp();
 #pragma unroll
         for (int c = 0; c < 8; ++c)
@@ -1003,7 +1009,7 @@ __device__ void export_tile_end(const KParams &p, uint32_t *acc, int t0, int R, 
                 const uint4 v = *reinterpret_cast<const uint4 *>(blk + row * 32 + ((c ^ (row & 7)) << 2));
 #pragma unroll
                 for (int s = 0; s < P; ++s)
-                    *reinterpret_cast<int4 *>(o + (size_t)(q * P + s) * p.n_rho) = fields4<P>(v, s);
+                    __stcs(reinterpret_cast<int4 *>(o + (size_t)(q * P + s) * p.n_rho), fields4<P>(v, s));
             }
         } else {
             for (int q = 0; q < 32; ++q) {
@@ -1024,6 +1030,8 @@ __device__ void export_tile_end(const KParams &p, uint32_t *acc, int t0, int R, 
         const int g = x / nr, j = rb + (x - g * nr);
         const int wr = g * 32 + lane;
         const uint32_t v = acc[(size_t)(g * (NB + kGuard) + j) * 32 + lane];
+        if (SUM)
+            sum = __dp4a(v, 0x01010101u, sum);
 #pragma unroll
         for (int s = 0; s < P; ++s) {
             const int t = t0 + wr * P + s;
@@ -1036,20 +1044,22 @@ __device__ void export_tile_end(const KParams &p, uint32_t *acc, int t0, int R, 
     const int nq = (p.n_rho - NB) >> 2;
     if (nq > 0) {
         const int nrows = min(R, p.n_theta - t0);
-        for (int x = threadIdx.x; x < nrows * nq; x += S::threads()) {
-            const int i = x / nq, k = x - i * nq;
-            const int b = 4 * k < lo ? 4 * k : 4 * k + NB;
-            int32_t *o = out + (size_t)(t0 + i) * p.n_rho + b;
-            if (vec) {
-                *reinterpret_cast<int4 *>(o) = make_int4(0, 0, 0, 0);
-            } else {
-                o[0] = 0;
-                o[1] = 0;
-                o[2] = 0;
-                o[3] = 0;
+        for (int i = warp; i < nrows; i += nw) {         // a row per warp step
+            int32_t *row = out + (size_t)(t0 + i) * p.n_rho;
+            for (int k = lane; k < nq; k += 32) {
+                int32_t *o = row + (4 * k < lo ? 4 * k : 4 * k + NB);
+                if (vec) {
+                    __stcs(reinterpret_cast<int4 *>(o), make_int4(0, 0, 0, 0));
+                } else {
+                    o[0] = 0;
+                    o[1] = 0;
+                    o[2] = 0;
+                    o[3] = 0;
+                }
             }
         }
     }
+    return sum;
 }
 
 // Zero the whole tile, guard columns included.
