@@ -526,8 +526,9 @@ int hough_find_noalloc(const hough_geometry *g, int n_theta, int n_rho,
  *     runs once over the batch, and each request's results are copied
  *     straight into its host buffers; the request then completes.
  * With n_slots > 1, requests that arrive while earlier batches are on the
- * GPU go into the next free slot at once (continuous batching), so their
- * copies and kernels overlap with the running ones.  Device buffers and
+ * GPU go into the next free slot (continuous batching), so their copies and
+ * kernels overlap with the running ones: at once when the queue holds a window
+ * per SM or more, else after up to 60 us, in which others may join them.  Device buffers and
  * pinned staging are allocated once, in hough_server_create, and stay
  * resident.  Each window's results are the same bits as hough_find gives it
  * alone: windows never interact.
@@ -549,13 +550,14 @@ typedef struct hough_server_config {
     int64_t slot_hits;     /* hits one batch can hold (>= 1)                            */
     int64_t max_queued;    /* requests waiting for a slot before submit says BUSY (>= 1) */
     hough_launch launch;   /* launch shape of the server's batches; all 0: chosen per
-                              batch, one CTA of 1024 threads per SM with 32-word-row
-                              tiles for batches of fewer than 2 windows per SM (the
-                              lowest latency), the context's shape when the server is
-                              created for larger ones (the library default, or what
-                              hough_set_launch or hough_autotune on representative
-                              windows chose: the highest throughput); the context's
-                              own shape is restored by hough_server_destroy */
+                              batch, the library's shapes for few windows (several
+                              CTAs per window, or large ones) for batches of fewer
+                              than 2 windows per SM (the lowest latency), the
+                              context's shape when the server is created for larger
+                              ones (the library default, or what hough_set_launch or
+                              hough_autotune on representative windows chose: the
+                              highest throughput); the context's own shape is
+                              restored by hough_server_destroy */
 } hough_server_config;
 
 /*

@@ -18,7 +18,7 @@ ROOT = os.path.dirname(PKG)
 SRC = os.path.join(PKG, "csrc", "hough_api.cu")
 SERVER_SRC = os.path.join(PKG, "csrc", "hough_server.cpp")
 FIND_SRCS = [os.path.join(PKG, "csrc", f"hough_find{k}.cu")
-             for k in ("", "_128", "_256", "_512", "_1024", "_fp64")]
+             for k in ("", "_128", "_256", "_512", "_1024", "_split", "_fp64")]
 UNITS = [SRC, *FIND_SRCS, SERVER_SRC]
 DEPS = [*UNITS, os.path.join(PKG, "csrc", "hough_kernels.cuh"),
         os.path.join(PKG, "csrc", "hough_encode.cuh"),

@@ -302,10 +302,10 @@ int resolve_launch(const hough_ctx *ctx, const hough_launch &in, hough_launch &o
 
 // The shape a find of n_windows windows and n_hits hits runs in: `base`, or,
 // when the shape was left to the library (automatic), one of other CTA sizes:
-//  - up to one window per SM: one CTA of 512 threads, of 1024 for more than
-//    kHeavyWindowHits hits per window on average (100 windows of 290 hits at
-//    512 x 512: 91, 72, 54 and 51 us with 128, 256, 512 and 1024 threads; one
-//    window of 142 hits 29, 27, 26 and 27 us);
+//  - up to one window per SM (those that split_for leaves): one CTA of 512
+//    threads, of 1024 for more than kHeavyWindowHits hits per window on average
+//    (100 windows of 290 hits at 512 x 512: 91, 72, 54 and 51 us with 128, 256,
+//    512 and 1024 threads);
 //  - up to two: two CTAs of 256 (300 windows of 290 hits: 103 and 80 us with
 //    128 and 256 threads);
 //  - where two CTAs fit on an SM: 128 threads each up to kLightWindowHits hits
@@ -433,7 +433,39 @@ struct Prepared {
     hough_launch l;
     size_t smem;
     unsigned grid;
+    int split;       // CTAs per window: 0 (the persistent kernels), or a cluster of them
 };
+
+// For a batch of few windows, when the shape was left to the library: CTAs per
+// window (a cluster), each with a share of its theta tiles, and their shape;
+// false for the persistent kernels.  As many CTAs per window as there are
+// tiles, up to eight, while all windows' CTAs are resident at once, at most two
+// to an SM (of 512 threads while they have an SM each, else 256).  Windows x
+// CTAs each, one CTA per window and this: 512 x 512, 1 of 177 hits 26.7 and
+// 16.5 us (x 4), 20 of 290 hits 47 and 29 (x 4), 100 of 290 hits 50 and 44
+// (x 2; x 4 42 but 100 of 70 hits 23, 18 x 2, 22 x 4), 300 of 290 hits 76 and 79;
+// 1024 x 1024, 1 of 960 hits 96 and 35 (x 8), 20 113 and 48 (x 8), 100 113 and
+// 110 (x 2).  The first CTA merges one kept list per CTA, so lists stay short.
+bool split_for(const hough_ctx *ctx, bool automatic, int64_t n_windows, int &split,
+               hough_launch &l, size_t &smem)
+{
+    if (!automatic || (ctx->th.flags & HOUGH_FLAG_FP64) || kept_region(ctx) > 64)
+        return false;
+    const int tiles = (ctx->n_theta + 127) / 128;
+    for (int c : {8, 4, 2}) {
+        if (c > tiles || n_windows * c > 2 * (int64_t)ctx->num_sms)
+            continue;
+        const bool one = n_windows * c <= ctx->num_sms;
+        if (resolve_launch(ctx, hough_launch{one ? 512 : 256, 32, 2048, one ? 1 : 2}, l, smem) != HOUGH_OK)
+            continue;
+        smem += (size_t)c * kept_region(ctx) * 8;
+        if (!smem_fits(ctx, smem, l.ctas_per_sm))
+            continue;
+        split = c;
+        return true;
+    }
+    return false;
+}
 
 // The find kernel of a context: fixed-point bins, or the FP64 variant.
 using FindKernel = void (*)(hk::KParams);
@@ -455,8 +487,19 @@ static FindKernel find_kernel_of(const hough_ctx *ctx, const hough_launch &l)
 
 // Resolve a launch shape, raise the kernel's shared-memory limit and size the
 // persistent grid (not stream operations, so this runs outside any capture).
-int prepare_find(hough_ctx *ctx, int64_t n_windows, const hough_launch &req, Prepared &pr)
+int prepare_find(hough_ctx *ctx, int64_t n_windows, const hough_launch &req, Prepared &pr,
+                 bool automatic = false)
 {
+    if (split_for(ctx, automatic, n_windows, pr.split, pr.l, pr.smem)) {
+        const void *fk = pr.l.threads == 256
+                             ? reinterpret_cast<const void *>(hk::find_split_kernel_256)
+                             : reinterpret_cast<const void *>(hk::find_split_kernel_512);
+        if (raise_smem_limit(fk, pr.smem) != HOUGH_OK)
+            return HOUGH_ERR_CUDA;
+        pr.grid = (unsigned)(n_windows * pr.split);
+        return HOUGH_OK;
+    }
+    pr.split = 0;
     int rc = resolve_launch(ctx, req, pr.l, pr.smem);
     if (rc != HOUGH_OK)
         return rc;
@@ -481,6 +524,27 @@ int enqueue_find(hough_ctx *ctx, const hough_hits *hits, const int64_t *offsets,
                  unsigned int *counter, const Prepared &pr)
 {
     hk::KParams p = make_params(ctx, hits, offsets, n_windows, out, counter, pr.l);
+    if (pr.split > 0) {
+        p.split = pr.split;
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = (unsigned)pr.split;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(pr.grid);
+        cfg.blockDim = dim3((unsigned)pr.l.threads);
+        cfg.dynamicSmemBytes = pr.smem;
+        cfg.stream = s;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        if (cudaLaunchKernelEx(&cfg, pr.l.threads == 256 ? hk::find_split_kernel_256 : hk::find_split_kernel_512, p) !=
+            cudaSuccess) {
+            cudaGetLastError();
+            return HOUGH_ERR_CUDA;
+        }
+        ctx->launches += 1;
+        return HOUGH_OK;
+    }
     find_kernel_of(ctx, pr.l)<<<pr.grid, pr.l.threads, pr.smem, s>>>(p);
     if (cudaGetLastError() != cudaSuccess)
         return HOUGH_ERR_CUDA;
@@ -490,10 +554,10 @@ int enqueue_find(hough_ctx *ctx, const hough_hits *hits, const int64_t *offsets,
 
 int launch_find(hough_ctx *ctx, const hough_hits *hits, const int64_t *offsets, int64_t n_windows,
                 const hough_tracks *out, cudaStream_t s, unsigned int *counter,
-                const hough_launch &req)
+                const hough_launch &req, bool automatic = false)
 {
     Prepared pr{};
-    int rc = prepare_find(ctx, n_windows, req, pr);
+    int rc = prepare_find(ctx, n_windows, req, pr, automatic);
     if (rc != HOUGH_OK)
         return rc;
     return enqueue_find(ctx, hits, offsets, n_windows, out, s, counter, pr);
@@ -769,7 +833,8 @@ int hough_find(hough_ctx *ctx, const hough_hits *hits, const int64_t *window_off
     if (!c)
         return fail(ctx, HOUGH_ERR_ALLOC);
     rc = launch_find(ctx, hits, window_offsets, n_windows, tracks_out, s, c,
-                     launch_for(ctx, ctx->launch, ctx->auto_launch, hits->n_hits, n_windows));
+                     launch_for(ctx, ctx->launch, ctx->auto_launch, hits->n_hits, n_windows),
+                     ctx->auto_launch);
     return fail(ctx, rc);
 }
 
@@ -1283,7 +1348,8 @@ int hough_find_host(hough_ctx *ctx, const hough_hits *hits, const int64_t *windo
     const int64_t n_chunks = n_windows >= 8192 ? 4 : 1;
     Prepared pr{};
     rc = prepare_find(ctx, (n_windows + n_chunks - 1) / n_chunks,
-                      launch_for(ctx, ctx->launch, ctx->auto_launch, hits->n_hits, n_windows), pr);
+                      launch_for(ctx, ctx->launch, ctx->auto_launch, hits->n_hits, n_windows), pr,
+                      ctx->auto_launch && n_chunks == 1);
     if (rc != HOUGH_OK)
         return fail(ctx, rc);
     auto clampH = [&](int64_t v) { return std::min<int64_t>(std::max<int64_t>(v, 0), H); };
@@ -1314,7 +1380,8 @@ int hough_find_host(hough_ctx *ctx, const hough_hits *hits, const int64_t *windo
         if (exp_acc)
             ct.acc = dt.acc + (size_t)w0 * ctx->n_theta * ctx->n_rho;
         Prepared pk = pr;
-        pk.grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(pr.grid, nw));
+        if (pk.split == 0)
+            pk.grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(pr.grid, nw));
         rc = enqueue_find(ctx, &dh, (const int64_t *)(base + o_off) + w0, nw, &ct, cs, ctr[k & 1], pk);
         if (rc != HOUGH_OK)
             return fail(ctx, rc);
@@ -1374,7 +1441,7 @@ int hough_plan_create(hough_ctx *ctx, const hough_hits *hits, const int64_t *win
     Prepared pr{};
     rc = n_windows > 0 ? prepare_find(ctx, n_windows,
                                       launch_for(ctx, ctx->launch, ctx->auto_launch,
-                                                 hits->n_hits, n_windows), pr)
+                                                 hits->n_hits, n_windows), pr, ctx->auto_launch)
                        : HOUGH_OK;
     if (rc != HOUGH_OK) {
         // nothing to capture

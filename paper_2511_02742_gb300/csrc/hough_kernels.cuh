@@ -45,6 +45,7 @@
 
 #include <cuda_runtime.h>
 #include <limits.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include "hough.h"
@@ -108,6 +109,7 @@ struct KParams {
     int lw;             // log2(WR)
     int hit_stage;      // HS
     int kp;             // top-k region (power of two >= max(32, max_peaks))
+    int split;          // CTAs per window (find_split_kernel)
     int tb, bb;         // bits of a theta row and of a rho bin in a 32-bit peak key
     unsigned acc_bytes; // shared memory of the tile (also the association's scratch)
 };
@@ -117,6 +119,7 @@ struct KParams {
 // the strides of the scan, the votes and the tables are immediate offsets.
 template <int NT, int WR>
 struct Shape {
+    static constexpr int kThreads = NT;
     static __device__ __forceinline__ int threads() { return NT ? NT : (int)blockDim.x; }
     static __device__ __forceinline__ int warps() { return threads() >> 5; }
     static __device__ __forceinline__ int word_rows(const KParams &p) { return WR ? WR : p.word_rows; }
@@ -153,14 +156,14 @@ __host__ __device__ inline SmemLayout smem_layout(size_t acc_bytes, int hit_stag
     off = align_up(off + (size_t)(kp + 256) * 8, 16);
     L.sel = off;                                    // peaks gathered to be ranked
     off = align_up(off + 2048, 16);
-    L.pk = off;                                     // the kept peaks' lines
-    off = align_up(off + (size_t)kp * 16, 16);
     L.hist = off;                                   // peak-vote histogram
     off = align_up(off + kHistBins * 4, 16);
     L.wtot = off;                                   // per-warp counts, two sets
     off = align_up(off + 64 * 4, 16);
-    L.list = off;                                   // flagged words, one list per warp
-    off = align_up(off + (size_t)n_warps * kListCap * 2, 16);
+    L.list = off;                                   // flagged quads, one list per warp; after
+    L.pk = off;                                     // the tiles the kept peaks' lines
+    const size_t list = (size_t)n_warps * kListCap * 2, pk = (size_t)kp * 16;
+    off = align_up(off + (list > pk ? list : pk), 16);
     L.total = off;
     return L;
 }
@@ -1084,14 +1087,16 @@ __device__ __forceinline__ void zero_tile(const KParams &p, uint32_t *tile)
 // CTA passes three block barriers in the common case: after the votes, at
 // the end of the peak search, and after the tile is zeroed.  tile: the tile's
 // words, guard columns included; carry: two rows of NB + 2 kGuard words.
+// [ta, tb): the theta rows of this CTA's tiles (a range that does not start at
+// row 0 starts on a tile and needs the window's hits staged at once).
 template <class S, int P, class Key, bool F64, bool SUM>
 __device__ __forceinline__ int process_tiles(const KParams &p, long long beg, int H, uint32_t *tile, int2 *stage,
                              uint32_t *carry, uint16_t *list, unsigned char *buf,
                              unsigned char *sel, int4 *pk, int *hist, int *wtot, WinScalars &ws,
-                             long long w, const Key *&keys, int &n_top)
+                             long long w, int ta, int tb, const Key *&keys, int &n_top)
 {
     const int WR = S::word_rows(p), R = WR * P, NB = p.n_b;
-    const int n_tiles = (p.n_theta + R - 1) / R;
+    const int n_tiles = (p.n_theta + R - 1) / R, k0 = ta / R, k1 = min(n_tiles, (tb + R - 1) / R);
     const bool single = H <= p.hit_stage;
     const int lane = threadIdx.x & 31;
     constexpr int lgP = P == 4 ? 2 : (P == 2 ? 1 : 0);
@@ -1110,7 +1115,30 @@ __device__ __forceinline__ int process_tiles(const KParams &p, long long beg, in
     if (single)
         nv = stage_hits<S>(p, beg, H, stage, wtot, ws);
 
-    for (int k = 0; k < n_tiles; ++k) {
+    if (k0 > 0 && k0 < k1) {
+        // the last two rows before the range, voted straight into the carry
+        const int t0 = k0 * R;
+        lo_prev = lo_row ? __ldg(lo_row + k0 - 1) : 0;
+        const unsigned cb = carry0 + (P == 1 || (k0 & 1) ? carry_row : 0u);
+        for (int j = threadIdx.x; j < NB; j += S::threads()) {
+            sts32(cb + (unsigned)j * 4u, 0u);
+            if (P == 1)
+                sts32(carry0 + (unsigned)j * 4u, 0u);
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < 2 * nv; i += S::threads()) {
+            const int2 h = stage[i >> 1];
+            const int up = i & 1, t = t0 - 1 - up;
+            const int j = rho_bin(h.x, h.y, __ldg(p.C + t), __ldg(p.S + t), p.D, p.K) - lo_prev;
+            if ((unsigned)j < (unsigned)NB) {
+                if constexpr (P == 1)
+                    red_add_shared((up ? carry0 : cb) + (unsigned)j * 4u, 1u);
+                else
+                    red_add_shared(cb + (unsigned)j * 4u, 1u << ((P - 1 - up) * (32 / P)));
+            }
+        }
+    }
+    for (int k = k0; k < k1; ++k) {
         const int t0 = k * R;
         const bool last = k == n_tiles - 1;
         const bool fast = !F64 && p.in_range && t0 + R <= p.n_theta;
@@ -1373,7 +1401,7 @@ __device__ __forceinline__ bool find_window(const KParams &p, long long w, long 
     const int nv = process_tiles<S, P, Key, F64, SUM>(
         p, beg, H, tile, stage, reinterpret_cast<uint32_t *>(smem + L.carry),
         reinterpret_cast<uint16_t *>(smem + L.list) + warp * kListCap, smem + L.buf, smem + L.sel,
-        pk, hist, reinterpret_cast<int *>(smem + L.wtot), ws, w, keys, n_top);
+        pk, hist, reinterpret_cast<int *>(smem + L.wtot), ws, w, 0, p.n_theta, keys, n_top);
     if (SUM && nv == -2)
         return false;
     const int need = nw * (n_top + 2);
@@ -1458,6 +1486,192 @@ __device__ __forceinline__ void find_body(const KParams &p)
     }
 }
 
+// ---- one window over the CTAs of a cluster
+
+// What a CTA of a cluster publishes of its tiles.
+struct SplitOut {
+    int n_top;           // its best peaks, sorted, at `keys` (shared address)
+    unsigned keys;
+    int found;
+    unsigned flags;
+    int overflow;        // a byte counter overflowed (SUM)
+};
+
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// A word of CTA `rank`'s shared memory, at this CTA's address `addr`.
+__device__ __forceinline__ uint32_t ld_cluster32(unsigned addr, unsigned rank)
+{
+    uint32_t r, v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(r) : "memory");
+    return v;
+}
+
+// One window in the counter width P: every CTA of the cluster takes its share
+// of the 128-row tiles (the first all of them if the hits do not fit in the
+// stage), the first CTA merges their sorted peaks -- a peak's place is its
+// place in its own list plus, by a search in each of the others, the number of
+// better ones there -- and makes the association.  False (in every CTA) when a
+// counter overflowed.
+template <class S, int P, class Key, bool SUM>
+__device__ __forceinline__ bool split_window(const KParams &p, long long w, long long beg, int H,
+                                             unsigned rank, const SmemLayout &L,
+                                             unsigned char *smem, SplitOut &so, WinScalars &ws)
+{
+    constexpr int nw = S::kThreads / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int C = p.split;
+    uint32_t *tile = reinterpret_cast<uint32_t *>(smem + L.acc);
+    int2 *stage = reinterpret_cast<int2 *>(smem + L.stage);
+    int *hist = reinterpret_cast<int *>(smem + L.hist);
+    int4 *pk = reinterpret_cast<int4 *>(smem + L.pk);
+    const int n128 = (p.n_theta + 127) >> 7;
+    int ta = (int)rank * n128 / C * 128, tb = ((int)rank + 1) * n128 / C * 128;
+    if (H > p.hit_stage) {
+        ta = 0;
+        tb = rank == 0 ? n128 * 128 : 0;
+    }
+    reset_window<S>(p, hist, ws);
+    const Key *keys = nullptr;
+    int n_top = 0, nv = 0;
+    if (ta < tb)
+        nv = process_tiles<S, P, Key, false, SUM>(
+            p, beg, H, tile, stage, reinterpret_cast<uint32_t *>(smem + L.carry),
+            reinterpret_cast<uint16_t *>(smem + L.list) + warp * kListCap, smem + L.buf,
+            smem + L.sel, pk, hist, reinterpret_cast<int *>(smem + L.wtot), ws, w, ta, tb, keys,
+            n_top);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        so.overflow = SUM && nv == -2 ? 1 : 0;
+        so.n_top = so.overflow ? 0 : n_top;
+        so.keys = n_top > 0 ? (unsigned)__cvta_generic_to_shared(keys) : 0u;
+        so.found = ws.n_found;
+        so.flags = ws.flags;
+    }
+    cluster_sync();
+    const unsigned so_at = (unsigned)__cvta_generic_to_shared(&so);
+    if (SUM) {
+        const unsigned bad = lane < C ? ld_cluster32(so_at + offsetof(SplitOut, overflow), lane) : 0u;
+        if (__any_sync(0xffffffffu, bad != 0u)) {
+            cluster_sync();                  // every CTA has read it
+            return false;
+        }
+    }
+    // lane c of every warp: CTA c's counts; the lists to this CTA's memory
+    Key *lists = reinterpret_cast<Key *>(smem + L.total);
+    int n_c = 0, found = 0;
+    unsigned flags = 0u;
+    if (rank == 0) {
+        if (lane < C) {
+            n_c = (int)ld_cluster32(so_at + offsetof(SplitOut, n_top), lane);
+            found = (int)ld_cluster32(so_at + offsetof(SplitOut, found), lane);
+            flags = ld_cluster32(so_at + offsetof(SplitOut, flags), lane);
+        }
+        for (int c = warp; c < C; c += nw) {
+            const int n = __shfl_sync(0xffffffffu, n_c, c);
+            const unsigned at = ld_cluster32(so_at + offsetof(SplitOut, keys), c);
+            for (int i = lane; i < n; i += 32) {
+                if constexpr (sizeof(Key) == 4)
+                    lists[c * p.kp + i] = ld_cluster32(at + (unsigned)i * 4u, c);
+                else
+                    lists[c * p.kp + i] = (Key)ld_cluster32(at + (unsigned)i * 8u, c) |
+                                          (Key)ld_cluster32(at + (unsigned)i * 8u + 4u, c) << 32;
+            }
+        }
+    }
+    cluster_sync();                          // the others may leave
+    if (rank != 0)
+        return true;
+    const int total = (int)__reduce_add_sync(0xffffffffu, (unsigned)n_c);
+    found = (int)__reduce_add_sync(0xffffffffu, (unsigned)found);
+    flags = __reduce_or_sync(0xffffffffu, flags);
+    n_top = min(p.max_peaks, total);
+    Key *sorted = reinterpret_cast<Key *>(smem + L.sel);
+    for (int x0 = 0; x0 < C * p.kp; x0 += S::kThreads) {
+        const int x = x0 + (int)threadIdx.x, c = x / p.kp, i = x - c * p.kp;
+        const bool in = c < C && i < __shfl_sync(0xffffffffu, n_c, min(c, 31));   // c is the warp's
+        const Key key = in ? lists[x] : (Key)0;
+        int r = i;
+        for (int o = 0; o < C; ++o) {
+            const int n = __shfl_sync(0xffffffffu, n_c, o);
+            if (o == c)
+                continue;
+            int lo = 0, hi = n;              // better peaks of CTA o
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (lists[o * p.kp + mid] < key)
+                    lo = mid + 1;
+                else
+                    hi = mid;
+            }
+            r += lo;
+        }
+        if (in && r < n_top) {
+            const int t = key_theta(p, key), b = key_rho(p, key);
+            sorted[r] = key;
+            pk[r] = make_int4(__ldg(p.C + t), __ldg(p.S + t),
+                              (int)((unsigned)p.D - ((unsigned)(b - p.tol) << p.K)), t | b << 16);
+        }
+    }
+    const int need = nw * (n_top + 2);
+    int *scr = reinterpret_cast<int *>(tile);
+    const bool cats = H <= (int)(p.acc_bytes >> 2) - 2 * need;
+    associate<S, Key, false>(p, w, beg, H, n_top, sorted, pk, nv == H ? stage : nullptr,
+                             cats ? scr + 2 * need : nullptr, scr, scr + need);
+    if (threadIdx.x == 0) {
+        if (found > p.max_peaks)
+            flags |= HOUGH_WIN_PEAK_OVERFLOW;
+        p.status[w] = flags;
+        p.n_peaks[w] = n_top;
+        if (p.n_found)
+            p.n_found[w] = found;
+    }
+    return true;
+}
+
+// Batches of fewer windows than the SMs hold: p.split CTAs (a cluster) per
+// window.
+template <class S>
+__device__ __forceinline__ void split_body(const KParams &p)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ WinScalars ws;
+    __shared__ SplitOut so;
+    const SmemLayout L = smem_layout(p.acc_bytes, p.hit_stage, p.n_b, p.kp, S::kThreads / 32);
+    const long long w = blockIdx.x / p.split;
+    const unsigned rank = blockIdx.x % p.split;
+    for (int i = threadIdx.x; i < (int)(p.acc_bytes >> 4); i += S::kThreads)
+        reinterpret_cast<uint4 *>(smem + L.acc)[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = threadIdx.x; i < 2 * (p.n_b + 2 * kGuard); i += S::kThreads)
+        reinterpret_cast<uint32_t *>(smem + L.carry)[i] = 0u;
+    const long long beg = p.offsets[w], end = p.offsets[w + 1];
+    if (!(beg >= 0 && beg <= end && end <= p.n_hits && end - beg < (1ll << 30))) {
+        if (rank == 0 && threadIdx.x == 0) {
+            p.status[w] = HOUGH_WIN_BAD_OFFSETS;
+            p.n_peaks[w] = 0;
+            if (p.n_found)
+                p.n_found[w] = 0;
+        }
+        return;                              // the whole cluster
+    }
+    const int H = (int)(end - beg);
+    bool done = false;                       // the widths as in find_body
+    if (H <= 255)
+        done = split_window<S, 4, uint32_t, false>(p, w, beg, H, rank, L, smem, so, ws);
+    else if (H < 1 << (32 - p.tb - p.bb) && p.in_range && H <= 8 * p.n_b)
+        done = split_window<S, 4, uint32_t, true>(p, w, beg, H, rank, L, smem, so, ws);
+    if (!done) {
+        if (H <= 65534)
+            split_window<S, 2, unsigned long long, false>(p, w, beg, H, rank, L, smem, so, ws);
+        else
+            split_window<S, 1, unsigned long long, false>(p, w, beg, H, rank, L, smem, so, ws);
+    }
+}
+
 // The find kernels (instances of find_body), compiled in translation units of
 // their own so that they build in parallel (hough_find*.cu): find_kernel
 // (fixed point, any CTA size up to 1024 threads and any tile), its instances
@@ -1469,5 +1683,8 @@ __global__ void find_kernel_256(KParams p);
 __global__ void find_kernel_512(KParams p);
 __global__ void find_kernel_1024(KParams p);
 __global__ void find_kernel_fp64(KParams p);
+// One window per cluster (hough_find_split.cu).
+__global__ void find_split_kernel_256(KParams p);
+__global__ void find_split_kernel_512(KParams p);
 
 }  // namespace hk

@@ -116,12 +116,10 @@ struct hough_server {
     hough_ctx *ctx = nullptr;
     hough_server_config cfg{};
     hough_launch saved_launch{};     // the context's shape before the server
-    // shapes chosen per batch when the configuration leaves the shape open:
-    // the latency shape for batches of fewer than 2 windows per SM, else the
-    // context's default (throughput) shape
+    // with the configuration's shape left open: batches of fewer than 2
+    // windows per SM in the library's shapes for few windows, larger ones in
+    // the context's own
     bool per_batch = false;
-    hough_launch lat_launch{}, thr_launch{};
-    bool thr_auto = false;           // thr_launch was left to the library
     bool saved_auto = false;         // the context's flag before the server
     int max_peaks = 0;
     size_t in_cap = 0, out_cap = 0, stage_cap = 0;
@@ -201,9 +199,7 @@ int launch_slot(hough_server *s, Slot &sl)
     t.hit_track = reinterpret_cast<int32_t *>(sl.d_out + O.ht);
     t.track_hits = reinterpret_cast<int32_t *>(sl.d_out + O.th);
     if (s->per_batch)
-        s->ctx->launch = sl.W >= 2 * (int64_t)s->ctx->num_sms
-                             ? launch_for(s->ctx, s->thr_launch, s->thr_auto, sl.H, sl.W)
-                             : launch_for(s->ctx, s->lat_launch, true, sl.H, sl.W);
+        s->ctx->auto_launch = s->saved_auto || sl.W < 2 * (int64_t)s->ctx->num_sms;
     int rc = hough_find(s->ctx, &hits, reinterpret_cast<const int64_t *>(sl.d_in + L.off), sl.W,
                         &t, sl.stream);
     if (rc != HOUGH_OK)
@@ -420,27 +416,18 @@ int hough_server_create(hough_ctx *ctx, const hough_server_config *cfg, hough_se
     s->ctx = ctx;
     s->cfg = *cfg;
     s->max_peaks = ctx->th.max_peaks;
-    // the server's launch shape: as given, else chosen per batch: large CTAs,
-    // one or two per SM (launch_for), for batches of fewer than two windows
-    // per SM, so that they spread over every SM and each window has many
-    // warps; the context's own shape (the library's choice, or what
-    // hough_set_launch or hough_autotune chose for the workload) for larger
-    // ones
+    // the server's launch shape: as given, else chosen per batch: the
+    // library's shapes for few windows (several CTAs per window, or large
+    // ones, so that the batch spreads over every SM) for batches of fewer than
+    // two windows per SM, the context's own shape (the library's choice, or
+    // what hough_set_launch or hough_autotune chose for the workload) for
+    // larger ones
     s->saved_launch = ctx->launch;
     s->saved_auto = ctx->auto_launch;
-    s->thr_auto = ctx->auto_launch;
     hough_launch want = cfg->launch;
     if (want.threads == 0 && want.word_rows == 0 && want.hit_stage == 0 && want.ctas_per_sm == 0) {
-        const hough_launch lat{1024, 32, 2048, 1};
-        s->thr_launch = ctx->launch;
-        want = lat;
-        if (hough_set_launch(ctx, &want) != HOUGH_OK)
-            want = s->thr_launch;       // no room for the latency shape: one shape
-        else
-            s->per_batch = true;
-        s->lat_launch = ctx->launch;
-    }
-    if (hough_set_launch(ctx, &want) != HOUGH_OK) {
+        s->per_batch = true;
+    } else if (hough_set_launch(ctx, &want) != HOUGH_OK) {
         ctx->launch = s->saved_launch;
         ctx->auto_launch = s->saved_auto;
         delete s;

@@ -2,8 +2,8 @@
 bit against the oracle: window sizes around the 8-bit limit and the packed
 compares' free bit, lines of more hits than a byte counts (the window is
 redone in 16 bits), accumulators of one row, of a partial tile and of one row
-past a tile, every CTA size, tiles of several row groups, stores that overflow
-with ties, and thresholds past a counter's range."""
+past a tile, every CTA size, tiles of several row groups, several CTAs per
+window, stores that overflow with ties, and thresholds past a counter's range."""
 import numpy as np
 import pytest
 
@@ -95,3 +95,18 @@ def test_large_windows(hough):
     rng = np.random.default_rng(25)
     w = _windows([_random(rng, n) for n in (4000, 9000, 32800, 65534, 65535, 65600)])
     _check(hough, w, 128, 128, (None, (256, 32, 512, 2)), max_peaks=16)
+
+
+@pytest.mark.parametrize("n_theta,n_rho,windows", [(512, 512, 1), (512, 512, 70), (1024, 1024, 3),
+                                                   (1024, 1024, 30), (257, 200, 5), (700, 300, 40)])
+def test_one_window_over_several_ctas(hough, n_theta, n_rho, windows):
+    """Batches of few windows run with several CTAs per window: uneven shares
+    of tiles, empty windows, windows past the stage, byte overflows, and both
+    wider counters; with the accumulator exported on the small ones."""
+    rng = np.random.default_rng(n_theta + windows)
+    sizes = [300, 0, 2500, 1, 9000, 65600, 40, 256][:windows]
+    parts = [_random(rng, n) for n in sizes]
+    v, s = _random(rng, 60)
+    parts += [(np.r_[v, [7] * 300], np.r_[s, [900] * 300])] * (windows > 8)
+    parts += [_random(rng, 20 + 7 * k) for k in range(windows - len(parts))]
+    _check(hough, _windows(parts[:windows]), n_theta, n_rho, export=windows <= 5)
