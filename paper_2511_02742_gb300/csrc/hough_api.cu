@@ -73,10 +73,12 @@ static bool box_votes_in_range(const hough_geometry *g, int n_theta, int n_rho, 
 // nb[WR index]; lo_all: [WR index][log2 P][tile], tiles ceil(n_theta / 32)
 // apart.
 // bin_align, lo_align: other multiples for NB (where it stays below n_rho) and
-// for lo (a power of two that divides n_rho and bin_align).
+// for lo (a power of two that divides n_rho and bin_align).  lp_end: only the
+// tiles of log2 P below it.
 static void narrow_tiles(const hough_geometry *g, int nt, int nr, const int32_t *C,
                          const int32_t *S, long long D, int K, int nb_out[3],
-                         std::vector<int32_t> &lo_all, int bin_align = 4, int lo_align = 4)
+                         std::vector<int32_t> &lo_all, int bin_align = 4, int lo_align = 4,
+                         int lp_end = 3)
 {
     std::vector<long long> rlo(nt), rhi(nt);
     for (int t = 0; t < nt; ++t)
@@ -87,7 +89,7 @@ static void narrow_tiles(const hough_geometry *g, int nt, int nr, const int32_t 
         const int WR = 32 << wi;
         std::vector<long long> tlo((size_t)3 * stride), thi((size_t)3 * stride);
         long long nb = 4;
-        for (int lp = 0; lp < 3; ++lp) {
+        for (int lp = 0; lp < lp_end; ++lp) {
             const int R = WR << lp;
             for (int k = 0; k * R < nt; ++k) {
                 long long lo = LLONG_MAX, hi = LLONG_MIN;
@@ -104,18 +106,38 @@ static void narrow_tiles(const hough_geometry *g, int nt, int nr, const int32_t 
         nb = (nb + lo_align - 1 + bin_align - 1) / bin_align * bin_align;
         nb = std::min<long long>(nb, nr);
         nb_out[wi] = (int)nb;
-        for (int lp = 0; lp < 3; ++lp)
+        for (int lp = 0; lp < lp_end; ++lp)
             for (int k = 0; k * (WR << lp) < nt; ++k)
                 lo_all[(size_t)(wi * 3 + lp) * stride + k] = (int32_t)(std::min(
                     std::max(tlo[(size_t)lp * stride + k], 0LL), (long long)nr - nb) & ~(long long)(lo_align - 1));
     }
 }
 
+// Counters per word of the find's windows of up to 255 hits: four (128-row
+// tiles), or two where 64-row tiles leave a last half tile out: every tile
+// costs P votes a hit whether its rows exist or not, and shorter tiles reach
+// fewer bins.  (180 x 1000: 6 votes a hit instead of 8, 708 bins a row instead
+// of 788, two CTAs per SM instead of one: 267 -> 206 us per 3001 windows.)  From
+// 256 rows on the longer tiles' fewer scans weigh more.
+static int find_pmax(const hough_ctx *ctx)
+{
+    const int r = ctx->n_theta % 128;
+    return !(ctx->th.flags & HOUGH_FLAG_FP64) && ctx->n_theta <= 192 && r > 0 && r <= 64 ? 2 : 4;
+}
+
 // Bins a find tile stores per row for this word-row count.
+static int find_bins(const hough_ctx *ctx, int word_rows);
+
+// The same for tiles of every counter width.
 static int tile_bins(const hough_ctx *ctx, int word_rows)
 {
     const int wi = word_rows == 32 ? 0 : (word_rows == 64 ? 1 : 2);
     return ctx->tile_nb[wi] > 0 ? ctx->tile_nb[wi] : ctx->n_rho;
+}
+
+static int find_bins(const hough_ctx *ctx, int word_rows)
+{
+    return word_rows == 32 && ctx->find_nb > 0 ? ctx->find_nb : tile_bins(ctx, word_rows);
 }
 
 // SM count and shared-memory limits of device dev.
@@ -224,7 +246,7 @@ int kept_region(const hough_ctx *ctx)
 // for its counts and slots, one of each per warp and category.
 size_t acc_bytes_for(const hough_ctx *ctx, int word_rows, int threads)
 {
-    return hk::align_up(std::max(hk::tile_words(word_rows, tile_bins(ctx, word_rows)) * 4,
+    return hk::align_up(std::max(hk::tile_words(word_rows, find_bins(ctx, word_rows)) * 4,
                                  (size_t)(threads / 32) * (ctx->th.max_peaks + 2) * 8),
                         16);
 }
@@ -232,7 +254,7 @@ size_t acc_bytes_for(const hough_ctx *ctx, int word_rows, int threads)
 size_t find_smem(const hough_ctx *ctx, int word_rows, int hit_stage, int threads)
 {
     return hk::smem_layout(acc_bytes_for(ctx, word_rows, threads), hit_stage,
-                           tile_bins(ctx, word_rows), kept_region(ctx), threads / 32)
+                           find_bins(ctx, word_rows), kept_region(ctx), threads / 32)
         .total;
 }
 
@@ -303,34 +325,40 @@ int resolve_launch(const hough_ctx *ctx, const hough_launch &in, hough_launch &o
 // The shape a find of n_windows windows and n_hits hits runs in: `base`, or,
 // when the shape was left to the library (automatic), one of other CTA sizes:
 //  - up to one window per SM (those that split_for leaves): one CTA of 512
-//    threads, of 1024 for more than kHeavyWindowHits hits per window on average
+//    threads, of 1024 for more than 280 hits per window on average
 //    (100 windows of 290 hits at 512 x 512: 91, 72, 54 and 51 us with 128, 256,
 //    512 and 1024 threads);
 //  - up to two: two CTAs of 256 (300 windows of 290 hits: 103 and 80 us with
 //    128 and 256 threads);
-//  - where two CTAs fit on an SM: 128 threads each up to kLightWindowHits hits
-//    per window, 512 above kHeavyWindowHits (3000 windows at 1024 x 1024, 128
-//    / 256 / 512 threads: 142 hits 0.47 / 0.51 / 0.50 ms, 285 hits 0.73 / 0.73 /
-//    0.72, 570 hits 1.35 / 1.23 / 1.11, 960 hits 2.09 / 1.80 / 1.59).
-constexpr int64_t kLightWindowHits = 200, kHeavyWindowHits = 280;
-
+//  - where two CTAs fit on an SM: 128 threads each for light windows, 512 for
+//    heavier ones.  3000 windows at 1024 x 1024, 128 / 256 / 512 threads: 142
+//    hits 0.47 / 0.51 / 0.50 ms, 285 hits 0.73 / 0.73 / 0.72, 570 hits 1.35 /
+//    1.23 / 1.11, 960 hits 2.09 / 1.80 / 1.59; with fewer tiles to share them
+//    larger CTAs pay sooner: 300 x 700, 43 hits 0.144 / 0.153 / 0.152, 142 hits
+//    0.267 / 0.248 / 0.236; 180 x 1000, 142 hits 0.222 / 0.214 / 0.206.
 hough_launch launch_for(const hough_ctx *ctx, const hough_launch &base, bool automatic,
                         int64_t n_hits, int64_t n_windows)
 {
     if (!automatic || n_windows <= 0)
         return base;
-    const bool heavy = n_hits > kHeavyWindowHits * n_windows;
-    const bool light = n_hits <= kLightWindowHits * n_windows;
-    hough_launch want = base;
-    if (n_windows <= ctx->num_sms)
-        want = hough_launch{heavy ? 1024 : 512, 32, 2048, 1};
-    else if (n_windows <= 2 * (int64_t)ctx->num_sms)
-        want = hough_launch{256, 32, 1024, 2};
-    else if (base.ctas_per_sm == 2 && (heavy || light))
-        want = hough_launch{heavy ? 512 : 128, 32, base.hit_stage, 2};
+    const bool tall = ctx->n_theta > 512;
+    const int64_t light = tall ? 200 : 64, heavy = tall ? 280 : 64;
     hough_launch l{};
     size_t smem = 0;
-    return resolve_launch(ctx, want, l, smem) == HOUGH_OK ? l : base;
+    auto pick = [&](const hough_launch &want) { return resolve_launch(ctx, want, l, smem) == HOUGH_OK; };
+    if (n_windows <= ctx->num_sms)
+        return pick(hough_launch{n_hits > 280 * n_windows ? 1024 : 512, 32, 2048, 1}) ? l : base;
+    if (n_windows <= 2 * (int64_t)ctx->num_sms)
+        return pick(hough_launch{256, 32, 1024, 2}) ? l : base;
+    if (base.ctas_per_sm == 2) {
+        if (n_hits <= light * n_windows && pick(hough_launch{128, 32, base.hit_stage, 2}))
+            return l;
+        if (n_hits > heavy * n_windows &&
+            (pick(hough_launch{512, 32, base.hit_stage, 2}) ||
+             (n_hits <= 512 * n_windows && pick(hough_launch{512, 32, 1024, 2}))))
+            return l;
+    }
+    return base;
 }
 
 namespace {
@@ -416,8 +444,11 @@ hk::KParams make_params(const hough_ctx *ctx, const hough_hits *hits, const int6
     p.word_rows = l.word_rows;
     p.lw = l.word_rows == 32 ? 5 : (l.word_rows == 64 ? 6 : 7);
     const int wi = p.lw - 5;
-    p.n_b = narrow ? tile_bins(ctx, l.word_rows) : ctx->n_rho;
+    p.n_b = narrow ? find_bins(ctx, l.word_rows) : ctx->n_rho;
     p.lo_tab = narrow && ctx->d_lo ? ctx->d_lo + (size_t)wi * 3 * ctx->lo_stride : nullptr;
+    if (narrow && ctx->find_nb > 0 && l.word_rows == 32)
+        p.lo_tab = ctx->d_lo + (size_t)12 * ctx->lo_stride;
+    p.pmax = l.word_rows == 32 ? find_pmax(ctx) : 4;
     p.lo_stride = ctx->lo_stride;
     p.hit_stage = l.hit_stage;
     p.kp = kept_region(ctx);
@@ -451,7 +482,7 @@ bool split_for(const hough_ctx *ctx, bool automatic, int64_t n_windows, int &spl
 {
     if (!automatic || (ctx->th.flags & HOUGH_FLAG_FP64) || kept_region(ctx) > 64)
         return false;
-    const int tiles = (ctx->n_theta + 127) / 128;
+    const int rows = 32 * find_pmax(ctx), tiles = (ctx->n_theta + rows - 1) / rows;
     for (int c : {8, 4, 2}) {
         if (c > tiles || n_windows * c > 2 * (int64_t)ctx->num_sms)
             continue;
@@ -733,6 +764,14 @@ int hough_create(const hough_geometry *g, int n_theta, int n_rho, const hough_th
                          ctx->K, nb_acc, lo_acc, 32, ctx->n_rho % 32 == 0 ? 32 : 4);
         ctx->acc_nb = nb_acc[0];
         lo_all.insert(lo_all.end(), lo_acc.begin(), lo_acc.begin() + 3 * ctx->lo_stride);
+        if (find_pmax(ctx) == 2) {
+            int nb_find[3];
+            narrow_tiles(&ctx->g, ctx->n_theta, ctx->n_rho, ctx->C.data(), ctx->S.data(), ctx->D,
+                         ctx->K, nb_find, lo_acc, exported ? 32 : 4,
+                         exported && ctx->n_rho % 8 == 0 ? 8 : 4, 2);
+            ctx->find_nb = nb_find[0];
+            lo_all.insert(lo_all.end(), lo_acc.begin(), lo_acc.begin() + 3 * ctx->lo_stride);
+        }
         if (cudaMalloc(&ctx->d_lo, sizeof(int32_t) * lo_all.size()) != cudaSuccess) {
             hough_destroy(ctx);
             return HOUGH_ERR_ALLOC;
@@ -1065,7 +1104,7 @@ int hough_accumulate(hough_ctx *ctx, const hough_hits *hits, const int64_t *wind
     const hough_launch l{threads, 32, hit_stage, occ};
     hk::AccParams q{};
     q.k = make_params(ctx, hits, window_offsets, n_windows, &out, nullptr, l);
-    q.k.n_b = ctx->acc_nb;
+    q.k.n_b = ctx->acc_nb;                   // its own tiles
     q.k.lo_tab = ctx->d_lo + (size_t)9 * ctx->lo_stride;
     // parts of whole 128-row tiles, about six per resident CTA (each part
     // stages the window's hits again); whole windows where votes may miss the
@@ -1140,6 +1179,8 @@ int hough_find_iterative(hough_ctx *ctx, const hough_hits *hits, const int64_t *
     out.hit_track = hit_track;
     out.window_status = window_status;
     q.k = make_params(ctx, hits, window_offsets, n_windows, &out, nullptr, l);
+    q.k.n_b = nb;                            // tiles of every counter width
+    q.k.lo_tab = ctx->d_lo;
     q.max_tracks = max_tracks;
     q.tracks = reinterpret_cast<int4 *>(tracks);
     q.n_tracks = n_tracks;

@@ -24,6 +24,7 @@ struct hough_ctx {
     // bin of every tile, [word-row count][log2 P][tile], tile rows lo_stride
     // apart (null: every tile starts at bin 0)
     int tile_nb[3] = {0, 0, 0};
+    int find_nb = 0;              // the find's own where it uses 64-row tiles (else 0)
     int32_t *d_lo = nullptr;
     int lo_stride = 0;
     int32_t *d_C = nullptr, *d_S = nullptr;

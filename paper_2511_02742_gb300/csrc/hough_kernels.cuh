@@ -109,6 +109,8 @@ struct KParams {
     int lw;             // log2(WR)
     int hit_stage;      // HS
     int kp;             // top-k region (power of two >= max(32, max_peaks))
+    int pmax;           // counters per word of the find's small windows: 4, or 2 where
+                        // 64-row tiles fit n_theta better
     int split;          // CTAs per window (find_split_kernel)
     int tb, bb;         // bits of a theta row and of a rho bin in a 32-bit peak key
     unsigned acc_bytes; // shared memory of the tile (also the association's scratch)
@@ -1448,12 +1450,16 @@ __device__ __forceinline__ void find_body(const KParams &p)
             // tiles, and so half the scan, the zeroing and the barriers.
             const bool key32 = H < 1 << (32 - p.tb - p.bb);
             bool done = false;
-            if (H <= 255)
-                done = find_window<S, 4, uint32_t, F64>(p, w, beg, H, L, smem, ws);
-            else if (key32 && !F64 && p.in_range && H <= 8 * p.n_b)
-                done = find_window<S, 4, uint32_t, F64, !F64>(p, w, beg, H, L, smem, ws);
+            if (p.pmax == 4) {
+                if (H <= 255)
+                    done = find_window<S, 4, uint32_t, F64>(p, w, beg, H, L, smem, ws);
+                else if (key32 && !F64 && p.in_range && H <= 8 * p.n_b)
+                    done = find_window<S, 4, uint32_t, F64, !F64>(p, w, beg, H, L, smem, ws);
+            }
             if (!done) {
-                if (H <= 65534)
+                if (key32 && H <= 65534)
+                    find_window<S, 2, uint32_t, F64>(p, w, beg, H, L, smem, ws);
+                else if (H <= 65534)
                     find_window<S, 2, unsigned long long, F64>(p, w, beg, H, L, smem, ws);
                 else
                     find_window<S, 1, unsigned long long, F64>(p, w, beg, H, L, smem, ws);
@@ -1512,7 +1518,7 @@ __device__ __forceinline__ uint32_t ld_cluster32(unsigned addr, unsigned rank)
 }
 
 // One window in the counter width P: every CTA of the cluster takes its share
-// of the 128-row tiles (the first all of them if the hits do not fit in the
+// of the tiles (the first all of them if the hits do not fit in the
 // stage), the first CTA merges their sorted peaks -- a peak's place is its
 // place in its own list plus, by a search in each of the others, the number of
 // better ones there -- and makes the association.  False (in every CTA) when a
@@ -1529,11 +1535,11 @@ __device__ __forceinline__ bool split_window(const KParams &p, long long w, long
     int2 *stage = reinterpret_cast<int2 *>(smem + L.stage);
     int *hist = reinterpret_cast<int *>(smem + L.hist);
     int4 *pk = reinterpret_cast<int4 *>(smem + L.pk);
-    const int n128 = (p.n_theta + 127) >> 7;
-    int ta = (int)rank * n128 / C * 128, tb = ((int)rank + 1) * n128 / C * 128;
+    const int unit = 32 * p.pmax, units = (p.n_theta + unit - 1) / unit;
+    int ta = (int)rank * units / C * unit, tb = ((int)rank + 1) * units / C * unit;
     if (H > p.hit_stage) {
         ta = 0;
-        tb = rank == 0 ? n128 * 128 : 0;
+        tb = rank == 0 ? units * unit : 0;
     }
     reset_window<S>(p, hist, ws);
     const Key *keys = nullptr;
@@ -1660,12 +1666,17 @@ __device__ __forceinline__ void split_body(const KParams &p)
     }
     const int H = (int)(end - beg);
     bool done = false;                       // the widths as in find_body
-    if (H <= 255)
-        done = split_window<S, 4, uint32_t, false>(p, w, beg, H, rank, L, smem, so, ws);
-    else if (H < 1 << (32 - p.tb - p.bb) && p.in_range && H <= 8 * p.n_b)
-        done = split_window<S, 4, uint32_t, true>(p, w, beg, H, rank, L, smem, so, ws);
+    const bool key32 = H < 1 << (32 - p.tb - p.bb);
+    if (p.pmax == 4) {
+        if (H <= 255)
+            done = split_window<S, 4, uint32_t, false>(p, w, beg, H, rank, L, smem, so, ws);
+        else if (key32 && p.in_range && H <= 8 * p.n_b)
+            done = split_window<S, 4, uint32_t, true>(p, w, beg, H, rank, L, smem, so, ws);
+    }
     if (!done) {
-        if (H <= 65534)
+        if (key32 && H <= 65534)
+            split_window<S, 2, uint32_t, false>(p, w, beg, H, rank, L, smem, so, ws);
+        else if (H <= 65534)
             split_window<S, 2, unsigned long long, false>(p, w, beg, H, rank, L, smem, so, ws);
         else
             split_window<S, 1, unsigned long long, false>(p, w, beg, H, rank, L, smem, so, ws);
