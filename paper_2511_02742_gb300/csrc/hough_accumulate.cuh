@@ -77,7 +77,7 @@ __device__ __forceinline__ bool acc_tile(const KParams &p, long long w, long lon
 template <class S>
 __device__ __forceinline__ void accumulate_body(const AccParams &q)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
+    extern __shared__ __align__(128) unsigned char smem[];
     __shared__ WinScalars ws;
     __shared__ int wtot[64];
     __shared__ unsigned total;

@@ -210,7 +210,7 @@ __device__ unsigned long long iter_best(const KParams &p, uint32_t *acc, const i
 
 __global__ void __launch_bounds__(512, 1) iterative_tiles_kernel(IterParams q)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
+    extern __shared__ __align__(128) unsigned char smem[];
     __shared__ WinScalars ws;
     __shared__ unsigned long long red[16];
     __shared__ int wtot[32];
@@ -400,7 +400,7 @@ __device__ __forceinline__ void iter_body(const IterParams &q)
 {
     using S = Shape<NT, 32>;
     constexpr int nw = NT / 32;
-    extern __shared__ __align__(16) unsigned char smem[];
+    extern __shared__ __align__(128) unsigned char smem[];
     __shared__ WinScalars ws;
     __shared__ IterScalars is;
     __shared__ int wtot[32];

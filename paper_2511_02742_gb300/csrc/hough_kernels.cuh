@@ -376,17 +376,43 @@ __device__ __forceinline__ void vote_tile(const KParams &p, unsigned acc0, unsig
         }
     };
     const int np = nh >> 1;
-    const int4 *stage2 = reinterpret_cast<const int4 *>(stage);
+    auto each = [&](auto cast) {
+        const int4 *stage2 = reinterpret_cast<const int4 *>(stage);
 #pragma unroll 2
-    for (int h = h0; h < np; h += hstep) {
-        const int4 hv = stage2[h];
-        vote(hv.x, hv.y);
-        vote(hv.z, hv.w);
+        for (int h = h0; h < np; h += hstep) {
+            const int4 hv = stage2[h];
+            cast(hv.x, hv.y);
+            cast(hv.z, hv.w);
+        }
+        if ((nh & 1) && h0 == np % hstep) {     // the odd hit: to the warps that are a pair short
+            const int2 hv = stage[nh - 1];
+            cast(hv.x, hv.y);
+        }
+    };
+    if constexpr (FAST && P == 4 && S::kThreads >= 512) {
+        // The column's place folded into the sum: with its address over 128
+        // added to the bin, the sum shifted to K - 7 has the word's address in
+        // its upper bits (mod 2^32: they hold addresses below 2^(39 - K)) and
+        // the lane's place takes the lower seven -- a shift and one logic
+        // operation beside the two multiply-adds, none of them in their pipe,
+        // which bounds the votes where an SM has warps enough (high pileup in two
+        // CTAs of 512: 0.50 -> 0.48 us per window; four CTAs of 128 threads lost
+        // 4%, so they keep the plain form).
+        const unsigned base = col - 4u * (unsigned)lane;
+        if ((base & 127u) == 0u && base + nr * 128u <= 1u << (39 - K)) {
+            const unsigned Df = (unsigned)D + ((base >> 7) << K);
+            const int sh = K - 7;
+            each([&](int phi, int z) {
+#pragma unroll
+                for (int k = 0; k < P; ++k) {
+                    const unsigned v = (unsigned)phi * (unsigned)c[k] + (unsigned)z * (unsigned)s[k] + Df;
+                    red_add_shared(((v >> sh) & ~127u) | (4u * (unsigned)lane), 1u << (k * CW));
+                }
+            });
+            return;
+        }
     }
-    if ((nh & 1) && h0 == np % hstep) {         // the odd hit: to the warps that are a pair short
-        const int2 hv = stage[nh - 1];
-        vote(hv.x, hv.y);
-    }
+    each(vote);
     if (oor)
         atomicOr(&ws.flags, HOUGH_WIN_VOTE_OUT_OF_RANGE);
 }
@@ -756,6 +782,7 @@ __device__ __forceinline__ int find_peaks(const KParams &p, const TileView &tv,
     int n = 0;                       // listed quads (of that row group)
     int found = 0;
     unsigned sum = 0u;               // votes in the fields scanned
+    int seen = p.max_peaks;          // peaks stored when vk was last worked out
     Key kth = (Key)ws.kth;
     int vk = ws.vk;
     // reserve room for c peaks: the first place, or -1 when the store is full
@@ -912,6 +939,20 @@ __device__ __forceinline__ int find_peaks(const KParams &p, const TileView &tv,
                     return make_key<Key>(p, v, t + row, b);
                 };
                 int v;
+                // windows of 256 hits and more find hundreds of peaks per tile:
+                // as they are stored the bound rises, so take it from the
+                // histogram as it stands, not only at a merge (uneven heavy
+                // windows 427 -> 406 us; smaller windows lost 1%)
+                if constexpr (SUM) {
+                    const int stored = *reinterpret_cast<volatile int *>(&ws.n_buf);
+                    if (stored - seen >= p.max_peaks) {
+                        seen = stored;
+                        vk = vote_bound(p, st, ws);
+                        for (unsigned r = am; r != 0u; r &= r - 1u)
+                            if (quad_count<P>(cw, quad_row<P>(__ffs(r) - 1)) < vk)
+                                am &= ~(r & (0u - r));
+                    }
+                }
                 if (kth != (Key)~(Key)0)             // with vk votes, the k-th best may still be before it
                     for (unsigned r = am; r != 0u; r &= r - 1u)
                         if (key_of(r, v) >= kth)
@@ -948,6 +989,7 @@ __device__ __forceinline__ int find_peaks(const KParams &p, const TileView &tv,
         merge_peaks<S>(p, st, ws);
         kth = (Key)ws.kth;
         vk = ws.vk;
+        seen = p.max_peaks;
     }
 }
 
@@ -1420,7 +1462,7 @@ __device__ __forceinline__ bool find_window(const KParams &p, long long w, long 
 template <class S, bool F64>
 __device__ __forceinline__ void find_body(const KParams &p)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
+    extern __shared__ __align__(128) unsigned char smem[];
     __shared__ WinScalars ws;
     const int nw = S::warps();
     const SmemLayout L = smem_layout(p.acc_bytes, p.hit_stage, p.n_b, p.kp, nw);
@@ -1644,7 +1686,7 @@ __device__ __forceinline__ bool split_window(const KParams &p, long long w, long
 template <class S>
 __device__ __forceinline__ void split_body(const KParams &p)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
+    extern __shared__ __align__(128) unsigned char smem[];
     __shared__ WinScalars ws;
     __shared__ SplitOut so;
     const SmemLayout L = smem_layout(p.acc_bytes, p.hit_stage, p.n_b, p.kp, S::kThreads / 32);
