@@ -631,9 +631,11 @@ def _serving_leg(args, dev):
            f.alloc_outputs(pool.n_windows, pool.n_hits, device="cpu", pin=True).items()}
     launch = [int(x) for x in args.serve_launch.split(",")] if args.serve_launch else None
     launch_used = (dict(zip(("threads", "word_rows", "hit_stage", "ctas_per_sm"), launch))
-                   if launch else {"below 2 windows per SM": "1024 threads, 1 CTA per SM, 32 "
-                                   "word rows, 2048-hit stage",
-                                   "from 2 windows per SM": tuned or hough.hough_get_launch(f.ctx)})
+                   if launch else {"up to 1 window per SM": "a cluster of 2 to 4 CTAs per window, or "
+                                   "one CTA of 512 or 1024 threads, 32 word rows, 2048-hit stage",
+                                   "up to 2 windows per SM": "256 threads, 2 CTAs per SM, 32 word "
+                                   "rows, 1024-hit stage",
+                                   "above": tuned or hough.hough_get_launch(f.ctx)})
     srv = hough.Server(f, n_slots=4, slot_windows=4096, slot_hits=1 << 21, max_queued=1 << 16,
                        launch=launch)
     # half a second at the configured rate first, not reported: the first
@@ -700,10 +702,11 @@ def _flush_l2(buf):
 
 
 def find_kernel_source_sha256():
-    """sha256 of the find kernel's source: hough_kernels.cuh, then hough_find.cu."""
+    """sha256 of the find kernel's source: hough_kernels.cuh, then the file of its
+    instance for CTAs of 128 threads, hough_find_128.cu."""
     import hashlib
     h = hashlib.sha256()
-    for name in ("hough_kernels.cuh", "hough_find.cu"):
+    for name in ("hough_kernels.cuh", "hough_find_128.cu"):
         h.update(open(os.path.join(ROOT, "paper_2511_02742_gb300", "csrc", name), "rb").read())
     return h.hexdigest()
 
@@ -1178,19 +1181,17 @@ def run_ours(args):
 def _smem_atomic_peak_gops(args):
     """Shared-memory atomic throughput measured by the bench-side probe
     (conflict-free 32-bit adds, all SMs), or the unit-count figure if the probe
-    is off.  The ceiling is the form the vote loop issues: atom.shared.add with
-    the returned old value consumed; the no-return red.shared.add is measured
-    beside it."""
+    is off.  The ceiling is the form the vote loop issues: red.shared.add, with
+    no returned value."""
     nominal = 152 * 32 * 2.070   # SMs x banks x GHz: one 32-lane wavefront per clock per SM
     if args.no_probe:
         return {"value": round(nominal, 1), "source": "nominal: 152 SMs x 32 banks x 2.07 GHz"}
     try:
         import bench_probe
-        v = bench_probe.smem_atomic_gops("atom")
         r = bench_probe.smem_atomic_gops("red")
-        return {"value": round(v, 1),
-                "source": "measured: conflict-free atom.shared.add.u32 with the returned value "
-                          "consumed (the vote loop's op), bench_probe",
+        return {"value": round(r, 1),
+                "source": "measured: conflict-free red.shared.add.u32 with no returned value "
+                          "(the vote loop's op), bench_probe",
                 "red_no_return_gops": round(r, 1)}
     except Exception as e:  # pragma: no cover
         return {"value": round(nominal, 1), "source": f"nominal (probe failed: {e})"}

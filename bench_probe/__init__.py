@@ -48,8 +48,8 @@ def load():
 def smem_atomic_gops(op: str = "atom", iters: int = 4096, blocks_per_sm: int = 2,
                      threads: int = 1024) -> float:
     """Best of a few runs, in 10^9 shared atomics per second over the whole GPU.
-    op "atom": atom.shared.add.u32 with the old value consumed (the vote loop's
-    form); op "red": red.shared.add.u32 (no returned value)."""
+    op "atom": atom.shared.add.u32 with the old value consumed; op "red":
+    red.shared.add.u32, no returned value (the vote loop's form)."""
     lib = load()
     best = 0.0
     for _ in range(3):

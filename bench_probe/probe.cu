@@ -5,11 +5,9 @@
 // a warp always hit 32 distinct banks (no bank conflict, no same-address
 // conflict): the best case the vote loop's layout aims for.  Two forms of the
 // 32-bit add are measured, each written as the instruction itself:
-//   op 0: atom.shared.add.u32 with the returned old value consumed -- the
-//         form the find kernel's vote loop issues (the old value tells it
-//         when a bin reaches the vote threshold);
-//   op 1: red.shared.add.u32, no returned value -- the form of the
-//         accumulator-only kernel.
+//   op 0: atom.shared.add.u32 with the returned old value consumed;
+//   op 1: red.shared.add.u32, no returned value -- the form the vote loops
+//         issue.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -37,7 +35,7 @@ __global__ void __launch_bounds__(1024) smem_atomic_probe(int iters, unsigned *s
                 asm volatile("red.shared.add.u32 [%0], 1;" :: "r"(a) : "memory");
         }
         if (OP == 0) {
-            // the returned values are consumed, as the vote loop consumes them
+            // the returned values are consumed
 #pragma unroll
             for (int k = 0; k < 8; ++k)
                 acc += old[k];
