@@ -605,7 +605,7 @@ unsigned int *counter_for(hough_ctx *ctx, cudaStream_t s)
     unsigned int *c = nullptr;
     if (cudaMalloc(&c, 2 * sizeof(unsigned int)) != cudaSuccess)
         return nullptr;
-    if (cudaMemset(c, 0, 2 * sizeof(unsigned int)) != cudaSuccess) {
+    if (cudaMemsetAsync(c, 0, 2 * sizeof(unsigned int), s) != cudaSuccess) {
         cudaFree(c);
         return nullptr;
     }
@@ -1184,7 +1184,11 @@ int hough_find_iterative(hough_ctx *ctx, const hough_hits *hits, const int64_t *
     q.max_tracks = max_tracks;
     q.tracks = reinterpret_cast<int4 *>(tracks);
     q.n_tracks = n_tracks;
-    q.work = counter_for(ctx, (cudaStream_t)stream);     // none while a capture cannot allocate it
+    // no counter in a capture: its graph may run beside other work of the stream
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const bool captured = stream && cudaStreamIsCapturing((cudaStream_t)stream, &cs) == cudaSuccess &&
+                          cs != cudaStreamCaptureStatusNone;
+    q.work = captured ? nullptr : counter_for(ctx, (cudaStream_t)stream);
     const long long grid = std::min<long long>(n_windows, (long long)ctx->num_sms * ctas);
     kernel<<<(unsigned)grid, threads, smem, (cudaStream_t)stream>>>(q);
     if (cudaGetLastError() != cudaSuccess)

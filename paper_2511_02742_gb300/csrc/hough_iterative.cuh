@@ -419,9 +419,9 @@ __device__ __forceinline__ void iter_body(const IterParams &q)
     const int32_t *lo_row = p.lo_tab ? p.lo_tab + 2 * p.lo_stride : nullptr;
     zero_tile<S>(p, tile);
     auto next = [&](long long w) {
+        __syncthreads();
         if (!q.work)
             return w + gridDim.x;
-        __syncthreads();
         if (threadIdx.x == 0)
             ws.next_w = (int)gridDim.x + (int)atomicAdd(q.work, 1u);
         __syncthreads();

@@ -47,3 +47,50 @@ def test_past_the_stage(hough):
                  [_random(rng, 30) for _ in range(30)])
     _check(hough, w, 256, 256, max_tracks=4)
     _check(hough, w, 512, 512, max_tracks=2)
+
+
+def test_captured_call_beside_the_stream(hough):
+    """A captured search replayed on one stream while the stream it was captured
+    on runs the same calls: every result is the oracle's."""
+    import torch
+    w = synth.generate(3000, ("poisson", 6, 0, 30), (100.0, 300.0), 0.02, seed=44)
+    f = hough.Finder(256, 256)
+    hits = dict(vane=torch.from_numpy(w.vane).cuda(), strip=torch.from_numpy(w.strip).cuda())
+    offs = torch.from_numpy(w.offsets).cuda()
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+
+    def outputs():
+        return (torch.zeros((w.n_windows, 16, 4), dtype=torch.int32, device="cuda"),
+                torch.zeros(w.n_windows, dtype=torch.int32, device="cuda"),
+                torch.zeros(w.n_hits, dtype=torch.int32, device="cuda"),
+                torch.zeros(w.n_windows, dtype=torch.int32, device="cuda"))
+
+    def call(out, stream):
+        hough.hough_find_iterative(f.ctx, f.hits_struct(hits), offs, w.n_windows, 16, *out,
+                                   stream=stream)
+
+    own, captured = outputs(), outputs()
+    found = f.alloc_outputs(w.n_windows, w.n_hits)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(a):
+        f.find(hits, offs, out=found, stream=a)      # the stream has its counter
+    a.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=a, capture_error_mode="thread_local"):
+        call(captured, a)
+    for _ in range(4):
+        with torch.cuda.stream(b):
+            g.replay()
+        call(own, a)
+        f.find(hits, offs, out=found, stream=a)
+    torch.cuda.synchronize()
+    phi, z = oracle.encode(synth.GEOMETRY, w.vane, w.strip)
+    rtr, rnt, rht = oracle.iterative(synth.GEOMETRY, 256, 256, phi, z, w.offsets, max_tracks=16)
+    for tr, nt, ht, st in (own, captured):
+        tr = tr.cpu().numpy().view(hough.ITER_DTYPE).reshape(w.n_windows, 16)
+        np.testing.assert_array_equal(nt.cpu().numpy(), rnt)
+        for k in range(w.n_windows):
+            np.testing.assert_array_equal(tr[k][:rnt[k]], rtr[k][:rnt[k]], err_msg=str(k))
+        np.testing.assert_array_equal(ht.cpu().numpy(), rht)
+        assert (st.cpu().numpy() == 0).all()
+    f.close()
