@@ -1234,7 +1234,7 @@ int hough_extend(hough_ctx *ctx, const hough_hits *hits, const int64_t *window_o
     const int caps[3] = {512, 1536, HOUGH_EXT_MAX_HITS};
     long long lo = -1;
     for (int pass = 0; pass < 3; ++pass) {
-        const size_t smem = hk::ext_smem_bytes(caps[pass], nv);
+        const size_t smem = hk::ext_smem_bytes(caps[pass], nv, ctx->th.max_peaks);
         if (smem > ctx->smem_optin)
             return fail(ctx, HOUGH_ERR_UNSUPPORTED_SHAPE);
         if (raise_smem_limit(reinterpret_cast<const void *>(hk::extend_kernel), smem) != HOUGH_OK)

@@ -25,11 +25,12 @@ struct ExtParams {
 // part), tag[cap] int16 (the hit's peak from the find step, -1 none, or
 // kExtClaimed + track once claimed), bucket[cap] int16 (hit indices grouped
 // by vane), group[cap] int16 (the find step's hits in track order),
-// bstart[n_vanes + 1] and bcur[n_vanes] int32, line[2 n_vanes + 4] int16 (the
-// track being built, in vane order).
-__host__ __device__ inline size_t ext_smem_bytes(int cap, int n_vanes)
+// bstart[n_vanes + 1] and bcur[n_vanes] int32, seed[max_peaks] uint32 (the least
+// bend << 12 | b of a peak's triplets before any hit was claimed, ~0 none),
+// line[2 n_vanes + 4] int16 (the track being built, in vane order).
+__host__ __device__ inline size_t ext_smem_bytes(int cap, int n_vanes, int max_peaks)
 {
-    return (size_t)cap * 12 + (size_t)(2 * n_vanes + 1) * 4 + (size_t)(2 * n_vanes + 4) * 2;
+    return (size_t)cap * 12 + (size_t)(2 * n_vanes + 1 + max_peaks) * 4 + (size_t)(2 * n_vanes + 4) * 2;
 }
 
 // The smallest key of the warp, (bend << 36) | (b << 24) | (a << 12) | c with
@@ -89,7 +90,8 @@ __global__ void __launch_bounds__(32) extend_kernel(ExtParams q)
     int16_t *group = bucket + cap;
     int32_t *bstart = reinterpret_cast<int32_t *>(group + cap);   // cap is a multiple of 8
     int32_t *bcur = bstart + nv + 1;
-    int16_t *line = reinterpret_cast<int16_t *>(bcur + nv);
+    unsigned *seed = reinterpret_cast<unsigned *>(bcur + nv);
+    int16_t *line = reinterpret_cast<int16_t *>(seed + p.max_peaks);
     const int vstep = p.box.vane_step;
 
     // this warp's windows, 32 looked at together: a launch skips the windows of
@@ -192,65 +194,132 @@ __global__ void __launch_bounds__(32) extend_kernel(ExtParams q)
             }
             __syncwarp();
 
-            // ---- the peaks in order
+            // ---- every peak's least triplet, a lane per place of the find's
+            // lists: the seed of the peak unless an earlier track takes its hits
             const hough_peak *pk = p.peaks + w * (long long)p.max_peaks;
-            int pos = 0, hbl = 0, ml = 0;
-            for (int pi = 0; pi < np; ++pi) {
-                if ((pi & 31) == 0 && pi + lane < np) {     // the next 32 peaks' groups, a lane each
-                    hbl = pk[pi + lane].hit_begin;
-                    ml = pk[pi + lane].n_hits;
-                }
-                const int hb = __shfl_sync(0xffffffffu, hbl, pi & 31);
-                const int m = __shfl_sync(0xffffffffu, ml, pi & 31);
-                const bool grp_ok = hb >= 0 && m >= 3 && (long long)hb + m <= H;
-                if (!grp_ok) {                  // fewer than three hits: no seed
-                    if (lane == 0)
-                        ext[pi] = make_int4(-1, 0, pos, -1);
+            for (int i = lane; i < np; i += 32)
+                seed[i] = 0xffffffffu;
+            __syncwarp();
+            for (int j = lane; j < H; j += 32) {
+                const int b = group[j];
+                const int pi = b < 0 ? -1 : tag[b];
+                if (pi < 0 || pi >= np || vs[b] < 0)
                     continue;
-                }
-                // seed: the smallest (bend, b, a, c) over the group's unclaimed triplets
-                unsigned long long best = ~0ull;
-                for (int j = lane; j < m; j += 32) {
-                    const int b = group[hb + j];
-                    if (b < 0 || tag[b] != pi)
+                const int hb = pk[pi].hit_begin, m = pk[pi].n_hits;
+                if (hb < 0 || m < 3 || (long long)hb + m > H || j < hb || j >= hb + m)
+                    continue;
+                const int vb = vs[b];
+                const int va = vb == 0 ? nv - 1 : vb - 1;
+                const int vc = vb + 1 == nv ? 0 : vb + 1;
+                const long long zb2 = 2LL * zs[b];
+                const int c0 = bstart[vc], c1 = bstart[vc + 1];
+                long long best = (long long)tol + 1;
+                for (int ia = bstart[va], ea = bstart[va + 1]; ia < ea; ++ia) {
+                    const int a = bucket[ia];
+                    if (tag[a] != pi)
                         continue;
-                    const int vb = vs[b];
-                    if (vb < 0)
-                        continue;
-                    const int va = vb == 0 ? nv - 1 : vb - 1;
-                    const int vc = vb + 1 == nv ? 0 : vb + 1;
-                    const long long zb2 = 2LL * zs[b];
-                    const int c0 = bstart[vc], c1 = bstart[vc + 1];
-                    for (int ia = bstart[va], ea = bstart[va + 1]; ia < ea; ++ia) {
-                        const int a = bucket[ia];
-                        if (tag[a] != pi)
+                    const long long za = zs[a];
+                    for (int ic = c0; ic < c1; ++ic) {
+                        const int c = bucket[ic];
+                        if (tag[c] != pi)
                             continue;
-                        const long long za = zs[a];
-                        for (int ic = c0; ic < c1; ++ic) {
-                            const int c = bucket[ic];
-                            if (tag[c] != pi)
-                                continue;
-                            long long bend = za - zb2 + zs[c];
-                            bend = bend < 0 ? -bend : bend;
-                            if (bend > tol)
-                                continue;
-                            const unsigned long long key = ((unsigned long long)bend << 36) |
-                                                           ((unsigned long long)b << 24) |
-                                                           ((unsigned long long)a << 12) |
-                                                           (unsigned long long)c;
-                            best = key < best ? key : best;
-                        }
+                        long long bend = za - zb2 + zs[c];
+                        bend = bend < 0 ? -bend : bend;
+                        best = bend < best ? bend : best;
                     }
                 }
-                best = ext_warp_min(best);
-                if (best == ~0ull) {
-                    if (lane == 0)
-                        ext[pi] = make_int4(-1, 0, pos, -1);
-                    continue;
+                if (best <= tol)
+                    atomicMin(&seed[pi], (unsigned)best << 12 | (unsigned)b);
+            }
+            __syncwarp();
+
+            // ---- the peaks in order
+            int pos = 0;
+            for (int p0 = 0; p0 < np; p0 += 32) {
+            const unsigned mine32 = p0 + lane < np ? seed[p0 + lane] : 0xffffffffu;
+            unsigned todo_p = __ballot_sync(0xffffffffu, mine32 != 0xffffffffu);
+            int done_p = 0;                     // peaks of these 32 whose entries are written
+            for (;;) {
+                const int kp = todo_p != 0u ? __ffs(todo_p) - 1 : 32;
+                if (lane >= done_p && lane < kp && p0 + lane < np)      // no seed
+                    ext[p0 + lane] = make_int4(-1, 0, pos, -1);
+                if (kp == 32)
+                    break;
+                todo_p &= todo_p - 1u;
+                done_p = kp + 1;
+                const int pi = p0 + kp;
+                const unsigned first_seed = __shfl_sync(0xffffffffu, mine32, kp);
+                int a, b = (int)(first_seed & 4095u), c;
+                unsigned ac = 0xffffffffu;      // the least a << 12 | c of that bend
+                if (tag[b] == pi) {
+                    const int vb = vs[b];
+                    const int va = vb == 0 ? nv - 1 : vb - 1;
+                    const int vc = vb + 1 == nv ? 0 : vb + 1;
+                    const long long zb2 = 2LL * zs[b], least = first_seed >> 12;
+                    const int c0 = bstart[vc], c1 = bstart[vc + 1];
+                    for (int ia = bstart[va] + lane, ea = bstart[va + 1]; ia < ea; ia += 32) {
+                        const int x = bucket[ia];
+                        if (tag[x] != pi)
+                            continue;
+                        const long long za = zs[x];
+                        for (int ic = c0; ic < c1; ++ic) {
+                            const int y = bucket[ic];
+                            const long long bend = za - zb2 + zs[y];
+                            if (tag[y] == pi && (bend == least || bend == -least))
+                                ac = min(ac, (unsigned)x << 12 | (unsigned)y);
+                        }
+                    }
+                    ac = __reduce_min_sync(0xffffffffu, ac);
                 }
-                const int b = (int)((best >> 24) & 4095u);
-                const int a = (int)((best >> 12) & 4095u);
-                const int c = (int)(best & 4095u);
+                if (ac != 0xffffffffu) {
+                    a = (int)(ac >> 12);
+                    c = (int)(ac & 4095u);
+                } else {
+                    // a hit of it is claimed: the least of the triplets left
+                    const int hb = pk[pi].hit_begin, m = pk[pi].n_hits;
+                    unsigned long long best = ~0ull;
+                    for (int j = lane; j < m; j += 32) {
+                        const int b = group[hb + j];
+                        if (b < 0 || tag[b] != pi)
+                            continue;
+                        const int vb = vs[b];
+                        if (vb < 0)
+                            continue;
+                        const int va = vb == 0 ? nv - 1 : vb - 1;
+                        const int vc = vb + 1 == nv ? 0 : vb + 1;
+                        const long long zb2 = 2LL * zs[b];
+                        const int c0 = bstart[vc], c1 = bstart[vc + 1];
+                        for (int ia = bstart[va], ea = bstart[va + 1]; ia < ea; ++ia) {
+                            const int a = bucket[ia];
+                            if (tag[a] != pi)
+                                continue;
+                            const long long za = zs[a];
+                            for (int ic = c0; ic < c1; ++ic) {
+                                const int c = bucket[ic];
+                                if (tag[c] != pi)
+                                    continue;
+                                long long bend = za - zb2 + zs[c];
+                                bend = bend < 0 ? -bend : bend;
+                                if (bend > tol)
+                                    continue;
+                                const unsigned long long key = ((unsigned long long)bend << 36) |
+                                                               ((unsigned long long)b << 24) |
+                                                               ((unsigned long long)a << 12) |
+                                                               (unsigned long long)c;
+                                best = key < best ? key : best;
+                            }
+                        }
+                    }
+                    best = ext_warp_min(best);
+                    if (best == ~0ull) {
+                        if (lane == 0)
+                            ext[pi] = make_int4(-1, 0, pos, -1);
+                        continue;
+                    }
+                    b = (int)((best >> 24) & 4095u);
+                    a = (int)((best >> 12) & 4095u);
+                    c = (int)(best & 4095u);
+                }
                 const int16_t mine = (int16_t)(kExtClaimed + pi);
                 int lo = nv + 1, hi = nv + 4;
                 if (lane == 0) {
@@ -314,6 +383,7 @@ __global__ void __launch_bounds__(32) extend_kernel(ExtParams q)
                     ext[pi] = make_int4(vs[line[lo]], cnt, pos, b);
                 pos += cnt;
                 __syncwarp();
+            }
             }
 
             // ---- per-hit track and the unclaimed hits in index order
