@@ -1232,22 +1232,25 @@ int hough_extend(hough_ctx *ctx, const hough_hits *hits, const int64_t *window_o
     // small stages for most windows (many warps per SM), then larger ones for
     // the windows above them
     const int caps[3] = {512, 1536, HOUGH_EXT_MAX_HITS};
+    // 8 |z| and tol stay below 2^31
+    const bool narrow_z = q.k.box.z_min > -(1 << 27) && q.k.box.z_end < 1 << 27;
+    void (*const kernel)(hk::ExtParams) = narrow_z ? hk::extend_kernel : hk::extend_kernel_wide;
     long long lo = -1;
     for (int pass = 0; pass < 3; ++pass) {
         const size_t smem = hk::ext_smem_bytes(caps[pass], nv, ctx->th.max_peaks);
         if (smem > ctx->smem_optin)
             return fail(ctx, HOUGH_ERR_UNSUPPORTED_SHAPE);
-        if (raise_smem_limit(reinterpret_cast<const void *>(hk::extend_kernel), smem) != HOUGH_OK)
+        if (raise_smem_limit(reinterpret_cast<const void *>(kernel), smem) != HOUGH_OK)
             return fail(ctx, HOUGH_ERR_CUDA);
         int occ = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, hk::extend_kernel, 32, smem) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, 32, smem) !=
                 cudaSuccess || occ < 1)
             return fail(ctx, HOUGH_ERR_CUDA);
         q.cap = caps[pass];
         q.lo = lo;
         q.flag_large = pass == 2;
         const long long grid = std::min<long long>(n_windows, (long long)ctx->num_sms * occ);
-        hk::extend_kernel<<<(unsigned)grid, 32, smem, (cudaStream_t)stream>>>(q);
+        kernel<<<(unsigned)grid, 32, smem, (cudaStream_t)stream>>>(q);
         if (cudaGetLastError() != cudaSuccess)
             return fail(ctx, HOUGH_ERR_CUDA);
         ctx->launches += 1;

@@ -48,17 +48,18 @@ __device__ __forceinline__ unsigned long long ext_warp_min(unsigned long long x)
 
 // The unclaimed hit of bucket [s0, s1) nearest to pred within tol, as the
 // key (|z - pred| << 13) | (z > pred) << 12 | hit: the minimum is the nearest,
-// then the lower z, then the lower index.  ~0u when there is none.
+// then the lower z, then the lower index.  ~0u when there is none.  Z: the type
+// that holds the prediction (7 |z|).
+template <class Z>
 __device__ __forceinline__ unsigned ext_nearest(const int32_t *zs, const int16_t *tag,
-                                                const int16_t *bucket, int s0, int s1,
-                                                long long pred, int tol)
+                                                const int16_t *bucket, int s0, int s1, Z pred, int tol)
 {
     unsigned best = 0xffffffffu;
     for (int i = s0 + (int)(threadIdx.x & 31); i < s1; i += 32) {
         const int h = bucket[i];
         if (tag[h] >= kExtClaimed)
             continue;
-        long long d = (long long)zs[h] - pred;
+        Z d = (Z)zs[h] - pred;
         const unsigned side = d > 0 ? 1u : 0u;
         d = d < 0 ? -d : d;
         if (d > tol)
@@ -77,7 +78,8 @@ __device__ __forceinline__ unsigned ext_nearest(const int32_t *zs, const int16_t
 // ten shuffles.  Not better: hits laid out in vane order (505 us: more work to
 // lay them out than the steps save), a 256-hit stage in front (40 warps per SM
 // need 48 registers and spill: 583 us).
-__global__ void __launch_bounds__(32) extend_kernel(ExtParams q)
+template <class Z>
+__device__ __forceinline__ void extend_body(const ExtParams &q)
 {
     extern __shared__ __align__(16) unsigned char ext_sm[];
     const KParams &p = q.k;
@@ -211,19 +213,19 @@ __global__ void __launch_bounds__(32) extend_kernel(ExtParams q)
                 const int vb = vs[b];
                 const int va = vb == 0 ? nv - 1 : vb - 1;
                 const int vc = vb + 1 == nv ? 0 : vb + 1;
-                const long long zb2 = 2LL * zs[b];
+                const Z zb2 = 2 * (Z)zs[b];
                 const int c0 = bstart[vc], c1 = bstart[vc + 1];
-                long long best = (long long)tol + 1;
+                Z best = (Z)tol + 1;
                 for (int ia = bstart[va], ea = bstart[va + 1]; ia < ea; ++ia) {
                     const int a = bucket[ia];
                     if (tag[a] != pi)
                         continue;
-                    const long long za = zs[a];
+                    const Z za = (Z)zs[a];
                     for (int ic = c0; ic < c1; ++ic) {
                         const int c = bucket[ic];
                         if (tag[c] != pi)
                             continue;
-                        long long bend = za - zb2 + zs[c];
+                        Z bend = za - zb2 + zs[c];
                         bend = bend < 0 ? -bend : bend;
                         best = bend < best ? bend : best;
                     }
@@ -255,16 +257,16 @@ __global__ void __launch_bounds__(32) extend_kernel(ExtParams q)
                     const int vb = vs[b];
                     const int va = vb == 0 ? nv - 1 : vb - 1;
                     const int vc = vb + 1 == nv ? 0 : vb + 1;
-                    const long long zb2 = 2LL * zs[b], least = first_seed >> 12;
+                    const Z zb2 = 2 * (Z)zs[b], least = (Z)(first_seed >> 12);
                     const int c0 = bstart[vc], c1 = bstart[vc + 1];
                     for (int ia = bstart[va] + lane, ea = bstart[va + 1]; ia < ea; ia += 32) {
                         const int x = bucket[ia];
                         if (tag[x] != pi)
                             continue;
-                        const long long za = zs[x];
+                        const Z za = (Z)zs[x];
                         for (int ic = c0; ic < c1; ++ic) {
                             const int y = bucket[ic];
-                            const long long bend = za - zb2 + zs[y];
+                            const Z bend = za - zb2 + zs[y];
                             if (tag[y] == pi && (bend == least || bend == -least))
                                 ac = min(ac, (unsigned)x << 12 | (unsigned)y);
                         }
@@ -287,18 +289,18 @@ __global__ void __launch_bounds__(32) extend_kernel(ExtParams q)
                             continue;
                         const int va = vb == 0 ? nv - 1 : vb - 1;
                         const int vc = vb + 1 == nv ? 0 : vb + 1;
-                        const long long zb2 = 2LL * zs[b];
+                        const Z zb2 = 2 * (Z)zs[b];
                         const int c0 = bstart[vc], c1 = bstart[vc + 1];
                         for (int ia = bstart[va], ea = bstart[va + 1]; ia < ea; ++ia) {
                             const int a = bucket[ia];
                             if (tag[a] != pi)
                                 continue;
-                            const long long za = zs[a];
+                            const Z za = (Z)zs[a];
                             for (int ic = c0; ic < c1; ++ic) {
                                 const int c = bucket[ic];
                                 if (tag[c] != pi)
                                     continue;
-                                long long bend = za - zb2 + zs[c];
+                                Z bend = za - zb2 + zs[c];
                                 bend = bend < 0 ? -bend : bend;
                                 if (bend > tol)
                                     continue;
@@ -331,11 +333,11 @@ __global__ void __launch_bounds__(32) extend_kernel(ExtParams q)
                 __syncwarp();
                 // forward: the parabola through the last three hits, one vane on
                 {
-                    long long z0 = zs[a], z1 = zs[b], z2 = zs[c];
+                    Z z0 = zs[a], z1 = zs[b], z2 = zs[c];
                     int v2 = vs[c];
                     while (hi - lo < nv) {
                         const int tv = v2 + 1 == nv ? 0 : v2 + 1;
-                        const unsigned key = ext_nearest(zs, tag, bucket, bstart[tv], bstart[tv + 1],
+                        const unsigned key = ext_nearest<Z>(zs, tag, bucket, bstart[tv], bstart[tv + 1],
                                                          3 * z2 - 3 * z1 + z0, tol);
                         if (key == 0xffffffffu)
                             break;
@@ -354,11 +356,11 @@ __global__ void __launch_bounds__(32) extend_kernel(ExtParams q)
                 }
                 // backward, from the seed's first hit
                 {
-                    long long z0 = zs[c], z1 = zs[b], z2 = zs[a];
+                    Z z0 = zs[c], z1 = zs[b], z2 = zs[a];
                     int v2 = vs[a];
                     while (hi - lo < nv) {
                         const int tv = v2 == 0 ? nv - 1 : v2 - 1;
-                        const unsigned key = ext_nearest(zs, tag, bucket, bstart[tv], bstart[tv + 1],
+                        const unsigned key = ext_nearest<Z>(zs, tag, bucket, bstart[tv], bstart[tv + 1],
                                                          3 * z2 - 3 * z1 + z0, tol);
                         if (key == 0xffffffffu)
                             break;
@@ -404,5 +406,9 @@ __global__ void __launch_bounds__(32) extend_kernel(ExtParams q)
         }
     }
 }
+
+// Predictions in 32 bits, and for geometries with z of 2^27 units and more.
+__global__ void __launch_bounds__(32) extend_kernel(ExtParams q) { extend_body<int>(q); }
+__global__ void __launch_bounds__(32) extend_kernel_wide(ExtParams q) { extend_body<long long>(q); }
 
 }  // namespace hk
