@@ -46,16 +46,16 @@ __device__ __forceinline__ unsigned long long ext_warp_min(unsigned long long x)
     return (unsigned long long)top << 24 | low;
 }
 
-// The unclaimed hit of bucket [s0, s1) nearest to pred within tol, as the
-// key (|z - pred| << 13) | (z > pred) << 12 | hit: the minimum is the nearest,
-// then the lower z, then the lower index.  ~0u when there is none.  Z: the type
-// that holds the prediction (7 |z|).
+// The unclaimed hit of bucket entries i, i + step, ... below s1 nearest to pred
+// within tol, as the key (|z - pred| << 13) | (z > pred) << 12 | hit: the
+// minimum is the nearest, then the lower z, then the lower index.  ~0u when
+// there is none.  Z: the type that holds the prediction (7 |z|).
 template <class Z>
-__device__ __forceinline__ unsigned ext_nearest(const int32_t *zs, const int16_t *tag,
-                                                const int16_t *bucket, int s0, int s1, Z pred, int tol)
+__device__ __forceinline__ unsigned ext_nearest(const int32_t *zs, const int16_t *tag, const int16_t *bucket,
+                                                int i, int s1, int step, Z pred, int tol)
 {
     unsigned best = 0xffffffffu;
-    for (int i = s0 + (int)(threadIdx.x & 31); i < s1; i += 32) {
+    for (; i < s1; i += step) {
         const int h = bucket[i];
         if (tag[h] >= kExtClaimed)
             continue;
@@ -67,7 +67,7 @@ __device__ __forceinline__ unsigned ext_nearest(const int32_t *zs, const int16_t
         const unsigned key = ((unsigned)d << 13) | (side << 12) | (unsigned)h;
         best = key < best ? key : best;
     }
-    return __reduce_min_sync(0xffffffffu, best);
+    return best;
 }
 
 // Bound: the dependent chain of a window's steps (a bucket's bounds, its hits, a
@@ -331,50 +331,97 @@ __device__ __forceinline__ void extend_body(const ExtParams &q)
                     line[lo + 2] = (int16_t)c;
                 }
                 __syncwarp();
-                // forward: the parabola through the last three hits, one vane on
+                // both ways at once, lanes 0 to 15 forward and 16 to 31 backward: the
+                // parabola through the last three hits, one vane on.  The two
+                // never meet while two vanes are free, so the hits are those of
+                // going forward first.
+                const int dir = lane >> 4;
+                bool any = true;
                 {
-                    Z z0 = zs[a], z1 = zs[b], z2 = zs[c];
-                    int v2 = vs[c];
-                    while (hi - lo < nv) {
-                        const int tv = v2 + 1 == nv ? 0 : v2 + 1;
-                        const unsigned key = ext_nearest<Z>(zs, tag, bucket, bstart[tv], bstart[tv + 1],
-                                                         3 * z2 - 3 * z1 + z0, tol);
-                        if (key == 0xffffffffu)
-                            break;
-                        const int h = (int)(key & 4095u);
-                        if (lane == 0) {
-                            tag[h] = mine;
-                            line[hi] = (int16_t)h;
+                    Z z0 = zs[dir ? c : a], z1 = zs[b], z2 = zs[dir ? a : c];
+                    int tv = vs[dir ? a : c];
+                    bool more = true;
+                    while (any && hi - lo + 2 <= nv) {
+                        tv = dir ? (tv == 0 ? nv - 1 : tv - 1) : (tv + 1 == nv ? 0 : tv + 1);
+                        const unsigned best = ext_nearest<Z>(zs, tag, bucket, bstart[tv] + (lane & 15),
+                                                             more ? bstart[tv + 1] : 0, 16, 3 * z2 - 3 * z1 + z0, tol);
+                        const unsigned kf = __reduce_min_sync(0xffffffffu, dir ? 0xffffffffu : best);
+                        const unsigned kb = __reduce_min_sync(0xffffffffu, dir ? best : 0xffffffffu);
+                        const unsigned key = dir ? kb : kf;
+                        hi += kf != 0xffffffffu ? 1 : 0;
+                        lo -= kb != 0xffffffffu ? 1 : 0;
+                        more = key != 0xffffffffu;
+                        if (more) {
+                            const int h = (int)(key & 4095u);
+                            if ((lane & 15) == 0) {
+                                tag[h] = mine;
+                                line[dir ? lo : hi - 1] = (int16_t)h;
+                            }
+                            z0 = z1;
+                            z1 = z2;
+                            z2 = zs[h];
                         }
-                        ++hi;
-                        z0 = z1;
-                        z1 = z2;
-                        z2 = zs[h];
-                        v2 = tv;
+                        any = (kf & kb) != 0xffffffffu;
                         __syncwarp();
                     }
                 }
-                // backward, from the seed's first hit
-                {
-                    Z z0 = zs[c], z1 = zs[b], z2 = zs[a];
-                    int v2 = vs[a];
-                    while (hi - lo < nv) {
-                        const int tv = v2 == 0 ? nv - 1 : v2 - 1;
-                        const unsigned key = ext_nearest<Z>(zs, tag, bucket, bstart[tv], bstart[tv + 1],
-                                                         3 * z2 - 3 * z1 + z0, tol);
-                        if (key == 0xffffffffu)
-                            break;
-                        const int h = (int)(key & 4095u);
-                        --lo;
-                        if (lane == 0) {
-                            tag[h] = mine;
-                            line[lo] = (int16_t)h;
+                if (any) {
+                    // they may meet: given back, and forward first
+                    for (int j = lo + lane; j < hi; j += 32)
+                        if (j < nv + 1 || j >= nv + 4) {
+                            const int h = line[j], ht = p.hit_track[beg + h];
+                            tag[h] = (int16_t)(ht >= 0 && ht < kExtClaimed ? ht : -1);
                         }
-                        z0 = z1;
-                        z1 = z2;
-                        z2 = zs[h];
-                        v2 = tv;
-                        __syncwarp();
+                    lo = nv + 1;
+                    hi = nv + 4;
+                    __syncwarp();
+                    // forward: the parabola through the last three hits, one vane on
+                    {
+                        Z z0 = zs[a], z1 = zs[b], z2 = zs[c];
+                        int v2 = vs[c];
+                        while (hi - lo < nv) {
+                            const int tv = v2 + 1 == nv ? 0 : v2 + 1;
+                            const unsigned key = __reduce_min_sync(
+                                0xffffffffu, ext_nearest<Z>(zs, tag, bucket, bstart[tv] + lane, bstart[tv + 1], 32,
+                                                            3 * z2 - 3 * z1 + z0, tol));
+                            if (key == 0xffffffffu)
+                                break;
+                            const int h = (int)(key & 4095u);
+                            if (lane == 0) {
+                                tag[h] = mine;
+                                line[hi] = (int16_t)h;
+                            }
+                            ++hi;
+                            z0 = z1;
+                            z1 = z2;
+                            z2 = zs[h];
+                            v2 = tv;
+                            __syncwarp();
+                        }
+                    }
+                    // backward, from the seed's first hit
+                    {
+                        Z z0 = zs[c], z1 = zs[b], z2 = zs[a];
+                        int v2 = vs[a];
+                        while (hi - lo < nv) {
+                            const int tv = v2 == 0 ? nv - 1 : v2 - 1;
+                            const unsigned key = __reduce_min_sync(
+                                0xffffffffu, ext_nearest<Z>(zs, tag, bucket, bstart[tv] + lane, bstart[tv + 1], 32,
+                                                            3 * z2 - 3 * z1 + z0, tol));
+                            if (key == 0xffffffffu)
+                                break;
+                            const int h = (int)(key & 4095u);
+                            --lo;
+                            if (lane == 0) {
+                                tag[h] = mine;
+                                line[lo] = (int16_t)h;
+                            }
+                            z0 = z1;
+                            z1 = z2;
+                            z2 = zs[h];
+                            v2 = tv;
+                            __syncwarp();
+                        }
                     }
                 }
                 __syncwarp();

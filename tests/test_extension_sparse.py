@@ -5,7 +5,9 @@ import numpy as np
 import pytest
 
 from paper_2511_02742_gb300 import synth
-from test_extension import G, TOL, _oracle
+
+from test_extension import G, TOL, _check, _oracle
+from test_find_edges import _windows
 
 pytestmark = pytest.mark.gpu
 
@@ -39,3 +41,24 @@ def test_few_windows_among_empty_ones(hough, n_windows):
     np.testing.assert_array_equal(out["ext_hits"].cpu().numpy()[:w.n_hits], rh)
     assert (out["window_status"].cpu().numpy()[:n_windows] == 0).all()
     f.close()
+
+
+@pytest.mark.parametrize("jitter", [0, 2, 7])
+def test_tracks_that_go_round(hough, jitter):
+    """Tracks on 3 to 40 of the 40 vanes, starting anywhere on the ring, alone
+    and beside a second one within reach: both ends are grown at once while
+    they cannot meet, and one after the other where they can."""
+    rng = np.random.default_rng(91 + jitter)
+    parts = []
+    for n in [3, 4, 5, 20, 35, 36, 37, 38, 39, 40, 40, 39, 38]:
+        for extra in (0, n // 2, 40):
+            v = (rng.integers(40) + np.arange(n)) % 40
+            u = (rng.integers(40) + np.arange(extra)) % 40
+            vane = np.r_[v, u]
+            strip = np.r_[1000 + rng.integers(-jitter, jitter + 1, n),
+                          1012 + rng.integers(-jitter, jitter + 1, extra)]
+            order = rng.permutation(len(vane))
+            parts.append((vane[order], strip[order]))
+    w = _windows(parts)
+    for tol in (TOL, 40 * 38):
+        _check(hough, w, 512, 512, tol=tol)
