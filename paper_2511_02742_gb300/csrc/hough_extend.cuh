@@ -71,13 +71,15 @@ __device__ __forceinline__ unsigned ext_nearest(const int32_t *zs, const int16_t
 }
 
 // Bound: the dependent chain of a window's steps (a bucket's bounds, its hits, a
-// warp minimum per vane) at 28 warps per SM, 0.66 instructions a cycle.  40001
-// windows of 86 hits: 530 us for the first launch and 13 + 27 us for the two that
-// find no window of their size -> 462, 5 and 6 us, by looking at 32 windows
-// together, by staging the groups and by two 32-bit minima per seed instead of
-// ten shuffles.  Not better: hits laid out in vane order (505 us: more work to
-// lay them out than the steps save), a 256-hit stage in front (40 warps per SM
-// need 48 registers and spill: 583 us).
+// warp minimum per vane) and its instructions (5.4 k) at 29 warps per SM, 0.64
+// instructions a cycle.  40001 windows of 86 hits, the first launch: 530 us ->
+// 462 by staging the groups and two 32-bit minima per seed instead of ten
+// shuffles, 412 by one pass for every peak's seed, 380 by predictions in 32
+// bits, 354 by growing both ends at once, 332 by one look at each bucket in
+// the seed pass; the launches that find no window of their size 13 + 27 -> 5 + 6
+// us by looking at 32 windows together.  Not better: hits laid out in vane
+// order (9% slower: more work to lay them out than the steps save), a 256-hit
+// stage in front (40 warps per SM need 48 registers and spill: 26% slower).
 template <class Z>
 __device__ __forceinline__ void extend_body(const ExtParams &q)
 {
@@ -161,12 +163,12 @@ __device__ __forceinline__ void extend_body(const ExtParams &q)
             }
             __syncwarp();
             {
-                // exclusive prefix over the vanes: lane l sums vanes [8l, 8l + 8)
-                const int v0 = lane * 8;
+                // exclusive prefix over the vanes: lane l sums vanes [l k, l k + k)
+                const int k = (nv + 31) >> 5;
+                const int v0 = min(lane * k, nv), v1 = min(v0 + k, nv);
                 int s = 0;
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    s += (v0 + j < nv) ? bcur[v0 + j] : 0;
+                for (int v = v0; v < v1; ++v)
+                    s += bcur[v];
                 int incl = s;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -175,15 +177,11 @@ __device__ __forceinline__ void extend_body(const ExtParams &q)
                         incl += y;
                 }
                 int run = incl - s;
-                __syncwarp();
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    if (v0 + j < nv) {
-                        const int c = bcur[v0 + j];
-                        bstart[v0 + j] = run;
-                        bcur[v0 + j] = run;
-                        run += c;
-                    }
+                for (int v = v0; v < v1; ++v) {
+                    const int c = bcur[v];
+                    bstart[v] = run;
+                    bcur[v] = run;
+                    run += c;
                 }
                 if (lane == 31)
                     bstart[nv] = incl;
@@ -215,19 +213,31 @@ __device__ __forceinline__ void extend_body(const ExtParams &q)
                 const int vc = vb + 1 == nv ? 0 : vb + 1;
                 const Z zb2 = 2 * (Z)zs[b];
                 const int c0 = bstart[vc], c1 = bstart[vc + 1];
+                // mostly one hit of the group stands on a vane
+                int n_c = 0;
+                Z zc = 0;
+                for (int ic = c0; ic < c1; ++ic) {
+                    const int c = bucket[ic];
+                    if (tag[c] == pi) {
+                        zc = (Z)zs[c];
+                        ++n_c;
+                    }
+                }
                 Z best = (Z)tol + 1;
-                for (int ia = bstart[va], ea = bstart[va + 1]; ia < ea; ++ia) {
+                for (int ia = bstart[va], ea = n_c > 0 ? bstart[va + 1] : ia; ia < ea; ++ia) {
                     const int a = bucket[ia];
                     if (tag[a] != pi)
                         continue;
                     const Z za = (Z)zs[a];
-                    for (int ic = c0; ic < c1; ++ic) {
+                    Z bend = za - zb2 + zc;
+                    bend = bend < 0 ? -bend : bend;
+                    best = bend < best ? bend : best;
+                    for (int ic = n_c > 1 ? c0 : c1; ic < c1; ++ic) {
                         const int c = bucket[ic];
-                        if (tag[c] != pi)
-                            continue;
-                        Z bend = za - zb2 + zs[c];
+                        bend = za - zb2 + zs[c];
                         bend = bend < 0 ? -bend : bend;
-                        best = bend < best ? bend : best;
+                        if (tag[c] == pi && bend < best)
+                            best = bend;
                     }
                 }
                 if (best <= tol)
@@ -238,201 +248,201 @@ __device__ __forceinline__ void extend_body(const ExtParams &q)
             // ---- the peaks in order
             int pos = 0;
             for (int p0 = 0; p0 < np; p0 += 32) {
-            const unsigned mine32 = p0 + lane < np ? seed[p0 + lane] : 0xffffffffu;
-            unsigned todo_p = __ballot_sync(0xffffffffu, mine32 != 0xffffffffu);
-            int done_p = 0;                     // peaks of these 32 whose entries are written
-            for (;;) {
-                const int kp = todo_p != 0u ? __ffs(todo_p) - 1 : 32;
-                if (lane >= done_p && lane < kp && p0 + lane < np)      // no seed
-                    ext[p0 + lane] = make_int4(-1, 0, pos, -1);
-                if (kp == 32)
-                    break;
-                todo_p &= todo_p - 1u;
-                done_p = kp + 1;
-                const int pi = p0 + kp;
-                const unsigned first_seed = __shfl_sync(0xffffffffu, mine32, kp);
-                int a, b = (int)(first_seed & 4095u), c;
-                unsigned ac = 0xffffffffu;      // the least a << 12 | c of that bend
-                if (tag[b] == pi) {
-                    const int vb = vs[b];
-                    const int va = vb == 0 ? nv - 1 : vb - 1;
-                    const int vc = vb + 1 == nv ? 0 : vb + 1;
-                    const Z zb2 = 2 * (Z)zs[b], least = (Z)(first_seed >> 12);
-                    const int c0 = bstart[vc], c1 = bstart[vc + 1];
-                    for (int ia = bstart[va] + lane, ea = bstart[va + 1]; ia < ea; ia += 32) {
-                        const int x = bucket[ia];
-                        if (tag[x] != pi)
-                            continue;
-                        const Z za = (Z)zs[x];
-                        for (int ic = c0; ic < c1; ++ic) {
-                            const int y = bucket[ic];
-                            const Z bend = za - zb2 + zs[y];
-                            if (tag[y] == pi && (bend == least || bend == -least))
-                                ac = min(ac, (unsigned)x << 12 | (unsigned)y);
-                        }
-                    }
-                    ac = __reduce_min_sync(0xffffffffu, ac);
-                }
-                if (ac != 0xffffffffu) {
-                    a = (int)(ac >> 12);
-                    c = (int)(ac & 4095u);
-                } else {
-                    // a hit of it is claimed: the least of the triplets left
-                    const int hb = pk[pi].hit_begin, m = pk[pi].n_hits;
-                    unsigned long long best = ~0ull;
-                    for (int j = lane; j < m; j += 32) {
-                        const int b = group[hb + j];
-                        if (b < 0 || tag[b] != pi)
-                            continue;
+                const unsigned mine32 = p0 + lane < np ? seed[p0 + lane] : 0xffffffffu;
+                unsigned todo_p = __ballot_sync(0xffffffffu, mine32 != 0xffffffffu);
+                int done_p = 0;                     // peaks of these 32 whose entries are written
+                for (;;) {
+                    const int kp = todo_p != 0u ? __ffs(todo_p) - 1 : 32;
+                    if (lane >= done_p && lane < kp && p0 + lane < np)      // no seed
+                        ext[p0 + lane] = make_int4(-1, 0, pos, -1);
+                    if (kp == 32)
+                        break;
+                    todo_p &= todo_p - 1u;
+                    done_p = kp + 1;
+                    const int pi = p0 + kp;
+                    const unsigned first_seed = __shfl_sync(0xffffffffu, mine32, kp);
+                    int a, b = (int)(first_seed & 4095u), c;
+                    unsigned ac = 0xffffffffu;      // the least a << 12 | c of that bend
+                    if (tag[b] == pi) {
                         const int vb = vs[b];
-                        if (vb < 0)
-                            continue;
                         const int va = vb == 0 ? nv - 1 : vb - 1;
                         const int vc = vb + 1 == nv ? 0 : vb + 1;
-                        const Z zb2 = 2 * (Z)zs[b];
+                        const Z zb2 = 2 * (Z)zs[b], least = (Z)(first_seed >> 12);
                         const int c0 = bstart[vc], c1 = bstart[vc + 1];
-                        for (int ia = bstart[va], ea = bstart[va + 1]; ia < ea; ++ia) {
-                            const int a = bucket[ia];
-                            if (tag[a] != pi)
+                        for (int ia = bstart[va] + lane, ea = bstart[va + 1]; ia < ea; ia += 32) {
+                            const int x = bucket[ia];
+                            if (tag[x] != pi)
                                 continue;
-                            const Z za = (Z)zs[a];
+                            const Z za = (Z)zs[x];
                             for (int ic = c0; ic < c1; ++ic) {
-                                const int c = bucket[ic];
-                                if (tag[c] != pi)
-                                    continue;
-                                Z bend = za - zb2 + zs[c];
-                                bend = bend < 0 ? -bend : bend;
-                                if (bend > tol)
-                                    continue;
-                                const unsigned long long key = ((unsigned long long)bend << 36) |
-                                                               ((unsigned long long)b << 24) |
-                                                               ((unsigned long long)a << 12) |
-                                                               (unsigned long long)c;
-                                best = key < best ? key : best;
+                                const int y = bucket[ic];
+                                const Z bend = za - zb2 + zs[y];
+                                if (tag[y] == pi && (bend == least || bend == -least))
+                                    ac = min(ac, (unsigned)x << 12 | (unsigned)y);
                             }
                         }
+                        ac = __reduce_min_sync(0xffffffffu, ac);
                     }
-                    best = ext_warp_min(best);
-                    if (best == ~0ull) {
-                        if (lane == 0)
-                            ext[pi] = make_int4(-1, 0, pos, -1);
-                        continue;
-                    }
-                    b = (int)((best >> 24) & 4095u);
-                    a = (int)((best >> 12) & 4095u);
-                    c = (int)(best & 4095u);
-                }
-                const int16_t mine = (int16_t)(kExtClaimed + pi);
-                int lo = nv + 1, hi = nv + 4;
-                if (lane == 0) {
-                    tag[a] = tag[b] = tag[c] = mine;
-                    line[lo] = (int16_t)a;
-                    line[lo + 1] = (int16_t)b;
-                    line[lo + 2] = (int16_t)c;
-                }
-                __syncwarp();
-                // both ways at once, lanes 0 to 15 forward and 16 to 31 backward: the
-                // parabola through the last three hits, one vane on.  The two
-                // never meet while two vanes are free, so the hits are those of
-                // going forward first.
-                const int dir = lane >> 4;
-                bool any = true;
-                {
-                    Z z0 = zs[dir ? c : a], z1 = zs[b], z2 = zs[dir ? a : c];
-                    int tv = vs[dir ? a : c];
-                    bool more = true;
-                    while (any && hi - lo + 2 <= nv) {
-                        tv = dir ? (tv == 0 ? nv - 1 : tv - 1) : (tv + 1 == nv ? 0 : tv + 1);
-                        const unsigned best = ext_nearest<Z>(zs, tag, bucket, bstart[tv] + (lane & 15),
-                                                             more ? bstart[tv + 1] : 0, 16, 3 * z2 - 3 * z1 + z0, tol);
-                        const unsigned kf = __reduce_min_sync(0xffffffffu, dir ? 0xffffffffu : best);
-                        const unsigned kb = __reduce_min_sync(0xffffffffu, dir ? best : 0xffffffffu);
-                        const unsigned key = dir ? kb : kf;
-                        hi += kf != 0xffffffffu ? 1 : 0;
-                        lo -= kb != 0xffffffffu ? 1 : 0;
-                        more = key != 0xffffffffu;
-                        if (more) {
-                            const int h = (int)(key & 4095u);
-                            if ((lane & 15) == 0) {
-                                tag[h] = mine;
-                                line[dir ? lo : hi - 1] = (int16_t)h;
+                    if (ac != 0xffffffffu) {
+                        a = (int)(ac >> 12);
+                        c = (int)(ac & 4095u);
+                    } else {
+                        // a hit of it is claimed: the least of the triplets left
+                        const int hb = pk[pi].hit_begin, m = pk[pi].n_hits;
+                        unsigned long long best = ~0ull;
+                        for (int j = lane; j < m; j += 32) {
+                            const int b = group[hb + j];
+                            if (b < 0 || tag[b] != pi)
+                                continue;
+                            const int vb = vs[b];
+                            if (vb < 0)
+                                continue;
+                            const int va = vb == 0 ? nv - 1 : vb - 1;
+                            const int vc = vb + 1 == nv ? 0 : vb + 1;
+                            const Z zb2 = 2 * (Z)zs[b];
+                            const int c0 = bstart[vc], c1 = bstart[vc + 1];
+                            for (int ia = bstart[va], ea = bstart[va + 1]; ia < ea; ++ia) {
+                                const int a = bucket[ia];
+                                if (tag[a] != pi)
+                                    continue;
+                                const Z za = (Z)zs[a];
+                                for (int ic = c0; ic < c1; ++ic) {
+                                    const int c = bucket[ic];
+                                    if (tag[c] != pi)
+                                        continue;
+                                    Z bend = za - zb2 + zs[c];
+                                    bend = bend < 0 ? -bend : bend;
+                                    if (bend > tol)
+                                        continue;
+                                    const unsigned long long key = ((unsigned long long)bend << 36) |
+                                                                   ((unsigned long long)b << 24) |
+                                                                   ((unsigned long long)a << 12) |
+                                                                   (unsigned long long)c;
+                                    best = key < best ? key : best;
+                                }
                             }
-                            z0 = z1;
-                            z1 = z2;
-                            z2 = zs[h];
                         }
-                        any = (kf & kb) != 0xffffffffu;
-                        __syncwarp();
+                        best = ext_warp_min(best);
+                        if (best == ~0ull) {
+                            if (lane == 0)
+                                ext[pi] = make_int4(-1, 0, pos, -1);
+                            continue;
+                        }
+                        b = (int)((best >> 24) & 4095u);
+                        a = (int)((best >> 12) & 4095u);
+                        c = (int)(best & 4095u);
                     }
-                }
-                if (any) {
-                    // they may meet: given back, and forward first
-                    for (int j = lo + lane; j < hi; j += 32)
-                        if (j < nv + 1 || j >= nv + 4) {
-                            const int h = line[j], ht = p.hit_track[beg + h];
-                            tag[h] = (int16_t)(ht >= 0 && ht < kExtClaimed ? ht : -1);
-                        }
-                    lo = nv + 1;
-                    hi = nv + 4;
+                    const int16_t mine = (int16_t)(kExtClaimed + pi);
+                    int lo = nv + 1, hi = nv + 4;
+                    if (lane == 0) {
+                        tag[a] = tag[b] = tag[c] = mine;
+                        line[lo] = (int16_t)a;
+                        line[lo + 1] = (int16_t)b;
+                        line[lo + 2] = (int16_t)c;
+                    }
                     __syncwarp();
-                    // forward: the parabola through the last three hits, one vane on
+                    // both ways at once, lanes 0 to 15 forward and 16 to 31 backward: the
+                    // parabola through the last three hits, one vane on.  The two
+                    // never meet while two vanes are free, so the hits are those of
+                    // going forward first.
+                    const int dir = lane >> 4;
+                    bool any = true;
                     {
-                        Z z0 = zs[a], z1 = zs[b], z2 = zs[c];
-                        int v2 = vs[c];
-                        while (hi - lo < nv) {
-                            const int tv = v2 + 1 == nv ? 0 : v2 + 1;
-                            const unsigned key = __reduce_min_sync(
-                                0xffffffffu, ext_nearest<Z>(zs, tag, bucket, bstart[tv] + lane, bstart[tv + 1], 32,
-                                                            3 * z2 - 3 * z1 + z0, tol));
-                            if (key == 0xffffffffu)
-                                break;
-                            const int h = (int)(key & 4095u);
-                            if (lane == 0) {
-                                tag[h] = mine;
-                                line[hi] = (int16_t)h;
+                        Z z0 = zs[dir ? c : a], z1 = zs[b], z2 = zs[dir ? a : c];
+                        int tv = vs[dir ? a : c];
+                        bool more = true;
+                        while (any && hi - lo + 2 <= nv) {
+                            tv = dir ? (tv == 0 ? nv - 1 : tv - 1) : (tv + 1 == nv ? 0 : tv + 1);
+                            const unsigned best = ext_nearest<Z>(zs, tag, bucket, bstart[tv] + (lane & 15),
+                                                                 more ? bstart[tv + 1] : 0, 16, 3 * z2 - 3 * z1 + z0, tol);
+                            const unsigned kf = __reduce_min_sync(0xffffffffu, dir ? 0xffffffffu : best);
+                            const unsigned kb = __reduce_min_sync(0xffffffffu, dir ? best : 0xffffffffu);
+                            const unsigned key = dir ? kb : kf;
+                            hi += kf != 0xffffffffu ? 1 : 0;
+                            lo -= kb != 0xffffffffu ? 1 : 0;
+                            more = key != 0xffffffffu;
+                            if (more) {
+                                const int h = (int)(key & 4095u);
+                                if ((lane & 15) == 0) {
+                                    tag[h] = mine;
+                                    line[dir ? lo : hi - 1] = (int16_t)h;
+                                }
+                                z0 = z1;
+                                z1 = z2;
+                                z2 = zs[h];
                             }
-                            ++hi;
-                            z0 = z1;
-                            z1 = z2;
-                            z2 = zs[h];
-                            v2 = tv;
+                            any = (kf & kb) != 0xffffffffu;
                             __syncwarp();
                         }
                     }
-                    // backward, from the seed's first hit
-                    {
-                        Z z0 = zs[c], z1 = zs[b], z2 = zs[a];
-                        int v2 = vs[a];
-                        while (hi - lo < nv) {
-                            const int tv = v2 == 0 ? nv - 1 : v2 - 1;
-                            const unsigned key = __reduce_min_sync(
-                                0xffffffffu, ext_nearest<Z>(zs, tag, bucket, bstart[tv] + lane, bstart[tv + 1], 32,
-                                                            3 * z2 - 3 * z1 + z0, tol));
-                            if (key == 0xffffffffu)
-                                break;
-                            const int h = (int)(key & 4095u);
-                            --lo;
-                            if (lane == 0) {
-                                tag[h] = mine;
-                                line[lo] = (int16_t)h;
+                    if (any) {
+                        // they may meet: given back, and forward first
+                        for (int j = lo + lane; j < hi; j += 32)
+                            if (j < nv + 1 || j >= nv + 4) {
+                                const int h = line[j], ht = p.hit_track[beg + h];
+                                tag[h] = (int16_t)(ht >= 0 && ht < kExtClaimed ? ht : -1);
                             }
-                            z0 = z1;
-                            z1 = z2;
-                            z2 = zs[h];
-                            v2 = tv;
-                            __syncwarp();
+                        lo = nv + 1;
+                        hi = nv + 4;
+                        __syncwarp();
+                        // forward: the parabola through the last three hits, one vane on
+                        {
+                            Z z0 = zs[a], z1 = zs[b], z2 = zs[c];
+                            int v2 = vs[c];
+                            while (hi - lo < nv) {
+                                const int tv = v2 + 1 == nv ? 0 : v2 + 1;
+                                const unsigned key = __reduce_min_sync(
+                                    0xffffffffu, ext_nearest<Z>(zs, tag, bucket, bstart[tv] + lane, bstart[tv + 1], 32,
+                                                                3 * z2 - 3 * z1 + z0, tol));
+                                if (key == 0xffffffffu)
+                                    break;
+                                const int h = (int)(key & 4095u);
+                                if (lane == 0) {
+                                    tag[h] = mine;
+                                    line[hi] = (int16_t)h;
+                                }
+                                ++hi;
+                                z0 = z1;
+                                z1 = z2;
+                                z2 = zs[h];
+                                v2 = tv;
+                                __syncwarp();
+                            }
+                        }
+                        // backward, from the seed's first hit
+                        {
+                            Z z0 = zs[c], z1 = zs[b], z2 = zs[a];
+                            int v2 = vs[a];
+                            while (hi - lo < nv) {
+                                const int tv = v2 == 0 ? nv - 1 : v2 - 1;
+                                const unsigned key = __reduce_min_sync(
+                                    0xffffffffu, ext_nearest<Z>(zs, tag, bucket, bstart[tv] + lane, bstart[tv + 1], 32,
+                                                                3 * z2 - 3 * z1 + z0, tol));
+                                if (key == 0xffffffffu)
+                                    break;
+                                const int h = (int)(key & 4095u);
+                                --lo;
+                                if (lane == 0) {
+                                    tag[h] = mine;
+                                    line[lo] = (int16_t)h;
+                                }
+                                z0 = z1;
+                                z1 = z2;
+                                z2 = zs[h];
+                                v2 = tv;
+                                __syncwarp();
+                            }
                         }
                     }
+                    __syncwarp();
+                    const int cnt = hi - lo;
+                    for (int j = lane; j < cnt; j += 32)
+                        q.ext_hits[beg + pos + j] = line[lo + j];
+                    if (lane == 0)
+                        ext[pi] = make_int4(vs[line[lo]], cnt, pos, b);
+                    pos += cnt;
+                    __syncwarp();
                 }
-                __syncwarp();
-                const int cnt = hi - lo;
-                for (int j = lane; j < cnt; j += 32)
-                    q.ext_hits[beg + pos + j] = line[lo + j];
-                if (lane == 0)
-                    ext[pi] = make_int4(vs[line[lo]], cnt, pos, b);
-                pos += cnt;
-                __syncwarp();
-            }
             }
 
             // ---- per-hit track and the unclaimed hits in index order

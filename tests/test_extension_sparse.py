@@ -4,8 +4,8 @@ every launch's size stand at the first, last and middle places of those looks.""
 import numpy as np
 import pytest
 
+import oracle
 from paper_2511_02742_gb300 import synth
-
 from test_extension import G, TOL, _check, _oracle
 from test_find_edges import _windows
 
@@ -62,3 +62,29 @@ def test_tracks_that_go_round(hough, jitter):
     w = _windows(parts)
     for tol in (TOL, 40 * 38):
         _check(hough, w, 512, 512, tol=tol)
+
+
+def test_wide_z(hough):
+    """z of 2^27 units and more, whose predictions need 64 bits."""
+    import torch
+    geom = dict(G, z_pitch_u=1 << 17, z_min_u=-(1 << 27), z_u_per_mm=G["z_u_per_mm"] * 3449)
+    w = synth.generate(60, ("poisson", 6, 0, 20), (100.0, 300.0), 0.05, seed=93)
+    tol = (1 << 19) - 1
+    f = hough.Finder(256, 256, geometry=geom, max_peaks=64)
+    hits = dict(vane=torch.from_numpy(w.vane).cuda(), strip=torch.from_numpy(w.strip).cuda())
+    o = torch.from_numpy(w.offsets).cuda()
+    found = f.find(hits, o)
+    out = f.extend(hits, o, found, tol)
+    torch.cuda.synchronize()
+    phi, z = oracle.encode(geom, w.vane, w.strip)
+    assert np.abs(z).max() > 1 << 26
+    ref = oracle.find_batch(geom, 256, 256, phi, z, w.offsets, max_peaks=64)
+    re, rt, rh = oracle.extend(geom, phi, z, w.offsets, ref, tol)
+    ext = out["tracks"].cpu().numpy().view(hough.EXT_DTYPE).reshape(w.n_windows, 64)
+    np.testing.assert_array_equal(found["n_peaks"].cpu().numpy(), ref["n_peaks"])
+    assert (rt >= 0).sum() > 100
+    for k in range(w.n_windows):
+        np.testing.assert_array_equal(ext[k][:ref["n_peaks"][k]], re[k][:ref["n_peaks"][k]])
+    np.testing.assert_array_equal(out["ext_track"].cpu().numpy()[:w.n_hits], rt)
+    np.testing.assert_array_equal(out["ext_hits"].cpu().numpy()[:w.n_hits], rh)
+    f.close()
