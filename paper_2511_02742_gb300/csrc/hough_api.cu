@@ -1230,13 +1230,15 @@ int hough_extend(hough_ctx *ctx, const hough_hits *hits, const int64_t *window_o
     q.ext_hits = out->ext_hits;
     q.status = out->window_status;
     // small stages for most windows (many warps per SM), then larger ones for
-    // the windows above them
+    // the windows above them; the largest alone where four of its warps per SM
+    // are one for every window (slicing, find and extension of 150 / 400 / 600
+    // windows: 98 / 103 / 109 us with three launches, 90 / 95 / 101 with one)
     const int caps[3] = {512, 1536, HOUGH_EXT_MAX_HITS};
     // 8 |z| and tol stay below 2^31
     const bool narrow_z = q.k.box.z_min > -(1 << 27) && q.k.box.z_end < 1 << 27;
     void (*const kernel)(hk::ExtParams) = narrow_z ? hk::extend_kernel : hk::extend_kernel_wide;
     long long lo = -1;
-    for (int pass = 0; pass < 3; ++pass) {
+    for (int pass = n_windows <= 4 * (int64_t)ctx->num_sms ? 2 : 0; pass < 3; ++pass) {
         const size_t smem = hk::ext_smem_bytes(caps[pass], nv, ctx->th.max_peaks);
         if (smem > ctx->smem_optin)
             return fail(ctx, HOUGH_ERR_UNSUPPORTED_SHAPE);

@@ -88,3 +88,37 @@ def test_wide_z(hough):
     np.testing.assert_array_equal(out["ext_track"].cpu().numpy()[:w.n_hits], rt)
     np.testing.assert_array_equal(out["ext_hits"].cpu().numpy()[:w.n_hits], rh)
     f.close()
+
+
+@pytest.mark.parametrize("n_windows", [300, 700, 5000])
+def test_too_large_beside_others(hough, n_windows):
+    """A window of more hits than a warp stages, flagged once and left without
+    tracks, among windows of all sizes; the others are the oracle's."""
+    import torch
+    big = synth.generate(1, 330, (100.0, 300.0), 0.05, seed=94)
+    w = synth.concat([synth.generate(2, t, (100.0, 300.0), 0.02, seed=95 + t) for t in (110, 50, 8)])
+    n, nb = np.diff(w.offsets), int(big.offsets[1])
+    assert nb > 4096
+    vane = np.concatenate([w.vane, big.vane])
+    strip = np.concatenate([w.strip, big.strip])
+    offs = np.full(n_windows + 1, w.n_hits, np.int64)
+    offs[:7] = w.offsets
+    offs[n_windows] = w.n_hits + nb
+    f = hough.Finder(256, 256, max_peaks=64)
+    hits = dict(vane=torch.from_numpy(vane).cuda(), strip=torch.from_numpy(strip).cuda())
+    o = torch.from_numpy(offs).cuda()
+    found = f.find(hits, o)
+    out = f.extend(hits, o, found, TOL)
+    torch.cuda.synchronize()
+    re, rt, rh, rnp = _oracle(w, 256, 256, TOL)
+    st = out["window_status"].cpu().numpy()
+    assert st[n_windows - 1] == hough.HOUGH_WIN_TOO_LARGE and (st[:n_windows - 1] == 0).all()
+    ext = out["tracks"].cpu().numpy().view(hough.EXT_DTYPE).reshape(n_windows, 64)
+    for k in range(6):
+        np.testing.assert_array_equal(ext[k][:rnp[k]], re[k][:rnp[k]])
+    et, eh = out["ext_track"].cpu().numpy(), out["ext_hits"].cpu().numpy()
+    np.testing.assert_array_equal(et[:w.n_hits], rt)
+    np.testing.assert_array_equal(eh[:w.n_hits], rh)
+    assert (et[w.n_hits:w.n_hits + nb] == -1).all()
+    np.testing.assert_array_equal(eh[w.n_hits:w.n_hits + nb], np.arange(nb))
+    f.close()
