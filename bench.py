@@ -633,7 +633,7 @@ def _serving_leg(args, dev):
     launch_used = (dict(zip(("threads", "word_rows", "hit_stage", "ctas_per_sm"), launch))
                    if launch else {"up to 1 window per SM": "a cluster of 2 to 4 CTAs per window, or "
                                    "one CTA of 512 or 1024 threads, 32 word rows, 2048-hit stage",
-                                   "up to 2 windows per SM": "256 threads, 2 CTAs per SM, 32 word "
+                                   "up to 2 windows per SM": "512 threads, 2 CTAs per SM, 32 word "
                                    "rows, 1024-hit stage",
                                    "above": tuned or hough.hough_get_launch(f.ctx)})
     srv = hough.Server(f, n_slots=4, slot_windows=4096, slot_hits=1 << 21, max_queued=1 << 16,

@@ -328,8 +328,10 @@ int resolve_launch(const hough_ctx *ctx, const hough_launch &in, hough_launch &o
 //    threads, of 1024 for more than 280 hits per window on average
 //    (100 windows of 290 hits at 512 x 512: 91, 72, 54 and 51 us with 128, 256,
 //    512 and 1024 threads);
-//  - up to two: two CTAs of 256 (300 windows of 290 hits: 103 and 80 us with
-//    128 and 256 threads);
+//  - up to two: two CTAs of 512, of 256 where those do not fit (300 windows,
+//    with the call's launch, 128 / 256 / 512 threads: 512 x 512, 70 hits
+//    47 / 48 / 48 us, 142 hits 70 / 67 / 60, 290 hits 105 / 96 / 90; 1024 x
+//    1024, 960 hits 237 with 256 and 211 with 512);
 //  - where two CTAs fit on an SM: 128 threads each for light windows, 512 for
 //    heavier ones.  3000 windows at 1024 x 1024, 128 / 256 / 512 threads: 142
 //    hits 0.47 / 0.51 / 0.50 ms, 285 hits 0.73 / 0.73 / 0.72, 570 hits 1.35 /
@@ -349,7 +351,7 @@ hough_launch launch_for(const hough_ctx *ctx, const hough_launch &base, bool aut
     if (n_windows <= ctx->num_sms)
         return pick(hough_launch{n_hits > 280 * n_windows ? 1024 : 512, 32, 2048, 1}) ? l : base;
     if (n_windows <= 2 * (int64_t)ctx->num_sms)
-        return pick(hough_launch{256, 32, 1024, 2}) ? l : base;
+        return pick(hough_launch{512, 32, 1024, 2}) || pick(hough_launch{256, 32, 1024, 2}) ? l : base;
     if (base.ctas_per_sm == 2) {
         if (n_hits <= light * n_windows && pick(hough_launch{128, 32, base.hit_stage, 2}))
             return l;
