@@ -12,7 +12,7 @@ struct SliceParams {
     const int32_t *in0, *in1;
     long long n, t0, step, n_windows, cap;
     int m;
-    int block;          // windows per CTA step, 32..kSliceBlock
+    int block;          // windows per CTA step, 8..kSliceBlock
     int32_t *out0, *out1;
     long long *out_index;
     long long *offsets;
@@ -75,8 +75,23 @@ __global__ void __launch_bounds__(256) slice_kernel(SliceParams q)
         bad |= __ldg(q.t + i) > __ldg(q.t + i + 1);
     if (__any_sync(full, bad) && lane == 0 && q.status)
         atomicOr(q.status, HOUGH_SLICE_UNSORTED);
-    // sum_{i<m} LB(i)
-    for (int i = warp; i < q.m; i += nw) {
+    const long long n_entries = q.n_windows + 1;          // offsets[0 .. n_windows]
+    const int B = q.block;
+    const long long first = (long long)blockIdx.x * B;
+    // the ends of the block [k0, kend): e = 0, 1
+    auto find_end = [&](long long k0, int e) {
+        const long long kk = e == 0 ? k0 : min(k0 + (long long)B, n_entries) - 1 + q.m;
+        const long long lb = warp_lower_bound(q.t, q.n, q.t0 + kk * q.step);
+        if (lane == 0)
+            ends[e] = lb;
+    };
+    // LB(i), i < m, and the ends of the CTA's first block, a warp each
+    for (int i = warp; i < q.m + 2; i += nw) {
+        if (i >= q.m) {
+            if (first < n_entries)
+                find_end(first, i - q.m);
+            continue;
+        }
         const long long lb = warp_lower_bound(q.t, q.n, q.t0 + (long long)i * q.step);
         if (lane == 0)
             base_s[i] = lb;
@@ -86,18 +101,14 @@ __global__ void __launch_bounds__(256) slice_kernel(SliceParams q)
     for (int i = 0; i < q.m; ++i)
         base += base_s[i];
 
-    const long long n_entries = q.n_windows + 1;          // offsets[0 .. n_windows]
-    const int B = q.block;
-    for (long long k0 = (long long)blockIdx.x * B; k0 < n_entries; k0 += (long long)gridDim.x * B) {
+    for (long long k0 = first; k0 < n_entries; k0 += (long long)gridDim.x * B) {
         const long long kend = min(k0 + (long long)B, n_entries);
         const int cnt = (int)(kend - k0) + q.m;            // LB(k0) .. LB(kend - 1 + m)
-        if (warp < 2) {
-            const long long kk = warp == 0 ? k0 : kend - 1 + q.m;
-            const long long lb = warp_lower_bound(q.t, q.n, q.t0 + kk * q.step);
-            if (lane == 0)
-                ends[warp] = lb;
+        if (k0 != first) {
+            if (warp < 2)
+                find_end(k0, warp);
+            __syncthreads();
         }
-        __syncthreads();
         const long long lo = ends[0];
         const long long hi = max(ends[1], lo);           // unsorted input: keep the range sane
         for (int x = threadIdx.x; x < cnt; x += blockDim.x)
