@@ -50,6 +50,9 @@ struct hough_ctx {
     // hough_accumulate's launch (threads per CTA, resident CTAs per SM),
     // worked out on its first call
     int acc_threads = 0, acc_occ = 0;
+    // find kernels whose static shared memory was looked at: 128 to 1024 threads,
+    // the others
+    bool static_smem_checked[5] = {false, false, false, false, false};
     int acc_nb = 0;               // bins its tiles store per row (lo: after the find's in d_lo)
     int cf_K[2] = {0, 0};
     long long cf_D[2] = {0, 0};
