@@ -1194,13 +1194,7 @@ int hough_find_iterative(hough_ctx *ctx, const hough_hits *hits, const int64_t *
     q.max_tracks = max_tracks;
     q.tracks = reinterpret_cast<int4 *>(tracks);
     q.n_tracks = n_tracks;
-    // no counter in a capture: its graph may run beside other work of the stream
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    const bool captured = stream && cudaStreamIsCapturing((cudaStream_t)stream, &cs) == cudaSuccess &&
-                          cs != cudaStreamCaptureStatusNone;
-    q.work = captured ? nullptr : counter_for(ctx, (cudaStream_t)stream);
-    const long long grid = std::min<long long>(n_windows, (long long)ctx->num_sms * ctas);
-    kernel<<<(unsigned)grid, threads, smem, (cudaStream_t)stream>>>(q);
+    kernel<<<(unsigned)n_windows, threads, smem, (cudaStream_t)stream>>>(q);
     if (cudaGetLastError() != cudaSuccess)
         return fail(ctx, HOUGH_ERR_CUDA);
     const long long grid_tiles = std::min<long long>(n_windows, (long long)ctx->num_sms);

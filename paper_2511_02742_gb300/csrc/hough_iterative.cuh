@@ -25,7 +25,6 @@ struct IterParams {
     int4 *tracks;               // [n_windows * max_tracks]: theta, rho, votes, n_hits
     int32_t *n_tracks;          // [n_windows]
     int cap_hits, cap_list;     // iterative_kernel: staged hits and listed bins
-    unsigned *work;             // next-window and finished-CTA counters, as the find's (null: windows in turn)
 };
 
 constexpr int kIterLeft = -1;   // n_tracks of a window left to iterative_tiles_kernel
@@ -381,8 +380,12 @@ __device__ __forceinline__ void iter_list(const KParams &p, unsigned acc0, int t
     }
 }
 
-// One window per CTA (grid-stride): the staged valid hits, one 8-bit tile of
-// 128 rows, and the list of the bins with at least `floor` votes (T, or more
+// One window per CTA, in a grid of all windows: CTAs start as others end, which
+// evens windows of different sizes out with no counter in memory that another
+// call, or a replayed capture, could be using (5000 windows of 142 hits, and of 1
+// to 40 tracks: 0.515 and 3.48 ms with persistent CTAs and a counter, 0.513 and
+// 3.48 so; 1e5 windows of 4 hits 0.384 and 0.368).  The staged valid hits, one 8-bit
+// tile of 128 rows, and the list of the bins with at least `floor` votes (T, or more
 // while the list cannot hold every bin >= T: its tracks are taken first, and
 // the hits left are voted again).  Left to iterative_tiles_kernel: windows of
 // more hits than are staged or than a key counts, of more than 255 hits where
@@ -417,253 +420,232 @@ __device__ __forceinline__ void iter_body(const IterParams &q)
     const unsigned acc0 = (unsigned)__cvta_generic_to_shared(tile) + kGuard * 128u;
     const int n_tiles = (p.n_theta + 127) / 128;
     const int32_t *lo_row = p.lo_tab ? p.lo_tab + 2 * p.lo_stride : nullptr;
-    zero_tile<S>(p, tile);
-    auto next = [&](long long w) {
-        __syncthreads();
-        if (!q.work)
-            return w + gridDim.x;
+    const long long w = blockIdx.x;
+    const long long beg = p.offsets[w], end = p.offsets[w + 1];
+    if (!(beg >= 0 && beg <= end && end <= p.n_hits && end - beg < (1ll << 30))) {
+        if (threadIdx.x == 0) {
+            p.status[w] = HOUGH_WIN_BAD_OFFSETS;
+            q.n_tracks[w] = 0;
+        }
+        return;
+    }
+    const int H = (int)(end - beg);
+    if (H > q.cap_hits || H >= 1 << (32 - shift) || (H > 255 && !(p.in_range && H <= 8 * NB))) {
         if (threadIdx.x == 0)
-            ws.next_w = (int)gridDim.x + (int)atomicAdd(q.work, 1u);
+            q.n_tracks[w] = kIterLeft;
+        return;
+    }
+    if (threadIdx.x == 0)
+        ws.flags = 0u;
+    // stage the valid hits with their window-local indices
+    int nv = 0;
+    for (int c0 = 0; c0 < H; c0 += NT) {
+        const int i = c0 + threadIdx.x;
+        int phi = 0, z = 0;
+        bool ok = false;
+        if (i < H) {
+            ok = load_hit(p, beg + i, phi, z);
+            p.hit_track[beg + i] = ok ? -1 : -2;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, ok);
+        if (lane == 0)
+            wtot[warp] = __popc(m);
         __syncthreads();
-        return (long long)ws.next_w;
-    };
-    for (long long w = blockIdx.x; w < p.n_windows; w = next(w)) {
-        const long long beg = p.offsets[w], end = p.offsets[w + 1];
-        if (!(beg >= 0 && beg <= end && end <= p.n_hits && end - beg < (1ll << 30))) {
+        const int c = lane < nw ? wtot[lane] : 0;
+        const int pos = nv + (int)__reduce_add_sync(0xffffffffu, (unsigned)(lane < warp ? c : 0)) + __popc(m & lt);
+        if (ok) {
+            stage[pos] = make_int2(phi, z);
+            sidx[pos] = (uint16_t)i;
+        }
+        nv += (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
+        __syncthreads();
+    }
+    int found = 0;
+    bool left = false;
+    while (nv > 0 && found < q.max_tracks) {
+        // vote every tile and list its bins >= floor
+        int floor = p.T;
+        if (threadIdx.x == 0) {
+            is.n_list = 0;
+            is.sum = 0u;
+            is.taken[0] = is.taken[1] = 0;
+        }
+        __syncthreads();
+        for (int k = 0; k < n_tiles && !left; ++k) {
+            const int t0 = k * 128;
+            const int lo = lo_row ? __ldg(lo_row + k) : 0;
+            zero_tile<S>(p, tile);
+            __syncthreads();
+            if (p.in_range && t0 + 128 <= p.n_theta)
+                vote_tile<S, 4, true>(p, acc0, 0u, stage, nv, t0, lo, ws);
+            else
+                vote_tile<S, 4, false>(p, acc0, 0u, stage, nv, t0, lo, ws);
+            int before = is.n_list;                  // of the tiles before (no one adds to it now)
+            __syncthreads();
+            iter_list<S>(p, acc0, t0, lo, floor, nv > 255, list, q.cap_list, is);
+            __syncthreads();
+            while (is.n_list > q.cap_list) {
+                // raise the floor until half the list is free, drop what
+                // falls below it, and list the tile again
+                for (int i = threadIdx.x; i < 64; i += NT)
+                    hist[i] = 0;
+                __syncthreads();
+                for (int i = threadIdx.x; i < q.cap_list; i += NT)
+                    atomicAdd(&hist[min((int)(list[i] >> shift), 63)], 1);
+                __syncthreads();
+                int n = 0, v = 64;
+                while (v > 0 && n + hist[v - 1] <= q.cap_list / 2)
+                    n += hist[--v];
+                floor = max(floor + 1, v);
+                left = left || v > 63;               // too many to tell apart
+                __syncthreads();
+                if (warp == 0) {
+                    int m = 0;
+                    for (int i0 = 0; i0 < before; i0 += 32) {
+                        const uint32_t key = i0 + lane < before ? list[i0 + lane] : 0u;
+                        const unsigned mk = __ballot_sync(0xffffffffu, (int)(key >> shift) >= floor);
+                        if (mk >> lane & 1u)
+                            list[m + __popc(mk & lt)] = key;
+                        m += __popc(mk);
+                        __syncwarp();
+                    }
+                    if (lane == 0)
+                        is.n_list = m;
+                }
+                __syncthreads();
+                before = is.n_list;
+                __syncthreads();
+                iter_list<S>(p, acc0, t0, lo, floor, false, list, q.cap_list, is);
+                __syncthreads();
+                if (left)
+                    break;
+            }
+        }
+        if (nv > 255 && is.sum != (unsigned)nv * (unsigned)p.n_theta)
+            left = true;                             // a byte overflowed
+        if (left)
+            break;
+        // this thread's hits still unassigned: bit k for hit k NT + threadIdx.x
+        unsigned alive = 0u;
+        for (int k = 0; k * NT + (int)threadIdx.x < nv; ++k)
+            alive |= 1u << k;
+        // each warp keeps its share of the list, in place, and drops the
+        // bins that fall below the floor
+        const int first = found, share = (is.n_list + nw - 1) / nw;
+        uint32_t *mine = list + warp * share;
+        int n = max(min(share, is.n_list - warp * share), 0);
+        int n_tk = 0;
+        for (;;) {
+            // take the last track's votes from the listed bins; the best left
+            uint32_t best = 0u;
+            int kept = 0;
+            for (int i0 = 0; i0 < n; i0 += 32) {
+                uint32_t key = i0 + lane < n ? mine[i0 + lane] : 0u;
+                if (n_tk > 0) {
+                    // a hit is in the bin when its sum is within 2^K of the bin's
+                    // first (mod 2^32: the sums span less than 2^32 - 2^K)
+                    const unsigned at = ((1u << shift) - 1u) - (key & ((1u << shift) - 1u));
+                    const int t = min((int)(at >> p.bb), p.n_theta - 1);
+                    const unsigned c = (unsigned)__ldg(p.C + t), s = (unsigned)__ldg(p.S + t);
+                    const unsigned d = (unsigned)p.D - ((at & ((1u << p.bb) - 1u)) << p.K);
+                    const unsigned one = 1u << p.K;
+                    const int4 *pair = reinterpret_cast<const int4 *>(tk);
+                    unsigned off = 0u;
+#pragma unroll 4
+                    for (int x = 0; x < n_tk >> 1; ++x) {
+                        const int4 h = pair[x];
+                        off += (unsigned)h.x * c + (unsigned)h.y * s + d < one ? 1u : 0u;
+                        off += (unsigned)h.z * c + (unsigned)h.w * s + d < one ? 1u : 0u;
+                    }
+                    if (n_tk & 1) {
+                        const int2 h = tk[n_tk - 1];
+                        off += (unsigned)h.x * c + (unsigned)h.y * s + d < one ? 1u : 0u;
+                    }
+                    key -= off << shift;
+                }
+                const bool ok = i0 + lane < n && (int)(key >> shift) >= floor;
+                const unsigned mk = __ballot_sync(0xffffffffu, ok);
+                if (ok)
+                    mine[kept + __popc(mk & lt)] = key;
+                kept += __popc(mk);
+                best = max(best, ok ? key : 0u);
+                __syncwarp();
+            }
+            n = kept;
+            best = __reduce_max_sync(0xffffffffu, best);
+            if (lane == 0)
+                wtot[warp] = (int)best;
+            __syncthreads();
+            best = __reduce_max_sync(0xffffffffu, lane < nw ? (unsigned)wtot[lane] : 0u);
+            const int votes = (int)(best >> shift);
+            if (best == 0u || votes < floor || found == q.max_tracks)
+                break;
+            const unsigned at = ((1u << shift) - 1u) - (best & ((1u << shift) - 1u));
+            const int bt = (int)(at >> p.bb), bb = (int)(at & ((1u << p.bb) - 1u));
+            const int c = __ldg(p.C + bt), s = __ldg(p.S + bt);
+            int &taken = is.taken[found & 1];
+            for (int k = 0; k * NT < nv; ++k) {
+                const int i = k * NT + (int)threadIdx.x;
+                bool take = false;
+                int2 h = make_int2(0, 0);
+                if (alive >> k & 1u) {
+                    h = stage[i];
+                    const int d = rho_bin(h.x, h.y, c, s, p.D, p.K) - bb;
+                    take = d <= p.tol && d >= -p.tol;
+                }
+                const unsigned m = __ballot_sync(0xffffffffu, take);
+                if (m != 0u) {
+                    int base = 0;
+                    if (lane == 0)
+                        base = atomicAdd(&taken, __popc(m));
+                    base = __shfl_sync(0xffffffffu, base, 0);
+                    if (take) {
+                        alive &= ~(1u << k);
+                        tk[base + __popc(m & lt)] = h;
+                        p.hit_track[beg + sidx[i]] = found;
+                    }
+                }
+            }
+            __syncthreads();
+            n_tk = taken;
             if (threadIdx.x == 0) {
-                p.status[w] = HOUGH_WIN_BAD_OFFSETS;
-                q.n_tracks[w] = 0;
+                q.tracks[(size_t)w * q.max_tracks + found] = make_int4(bt, bb, votes, n_tk);
+                is.taken[(found + 1) & 1] = 0;
             }
-            continue;
+            ++found;
         }
-        const int H = (int)(end - beg);
-        if (H > q.cap_hits || H >= 1 << (32 - shift) || (H > 255 && !(p.in_range && H <= 8 * NB))) {
-            if (threadIdx.x == 0)
-                q.n_tracks[w] = kIterLeft;
-            continue;
+        if (floor == p.T || found == q.max_tracks)
+            break;
+        if (found == first) {
+            left = true;                             // more equal bins than the list holds
+            break;
         }
-        __syncthreads();                                 // the last window's reads are over
-        if (threadIdx.x == 0)
-            ws.flags = 0u;
-        // stage the valid hits with their window-local indices
-        int nv = 0;
-        for (int c0 = 0; c0 < H; c0 += NT) {
-            const int i = c0 + threadIdx.x;
-            int phi = 0, z = 0;
-            bool ok = false;
-            if (i < H) {
-                ok = load_hit(p, beg + i, phi, z);
-                p.hit_track[beg + i] = ok ? -1 : -2;
-            }
-            const unsigned m = __ballot_sync(0xffffffffu, ok);
+        // the hits left, in order, for the next list
+        int kept = 0;
+        __syncthreads();
+        for (int k = 0; k * NT < nv; ++k) {
+            const int i = k * NT + (int)threadIdx.x;
+            const bool keep = alive >> k & 1u;
+            const int2 h = keep ? stage[i] : make_int2(0, 0);
+            const uint16_t ix = keep ? sidx[i] : (uint16_t)0;
+            const unsigned m = __ballot_sync(0xffffffffu, keep);
             if (lane == 0)
                 wtot[warp] = __popc(m);
             __syncthreads();
             const int c = lane < nw ? wtot[lane] : 0;
-            const int pos = nv + (int)__reduce_add_sync(0xffffffffu, (unsigned)(lane < warp ? c : 0)) + __popc(m & lt);
-            if (ok) {
-                stage[pos] = make_int2(phi, z);
-                sidx[pos] = (uint16_t)i;
+            const int pos = kept + (int)__reduce_add_sync(0xffffffffu, (unsigned)(lane < warp ? c : 0)) + __popc(m & lt);
+            if (keep) {
+                stage[pos] = h;
+                sidx[pos] = ix;
             }
-            nv += (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
+            kept += (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
             __syncthreads();
         }
-        int found = 0;
-        bool left = false;
-        while (nv > 0 && found < q.max_tracks) {
-            // vote every tile and list its bins >= floor
-            int floor = p.T;
-            if (threadIdx.x == 0) {
-                is.n_list = 0;
-                is.sum = 0u;
-                is.taken[0] = is.taken[1] = 0;
-            }
-            __syncthreads();
-            for (int k = 0; k < n_tiles && !left; ++k) {
-                const int t0 = k * 128;
-                const int lo = lo_row ? __ldg(lo_row + k) : 0;
-                if (p.in_range && t0 + 128 <= p.n_theta)
-                    vote_tile<S, 4, true>(p, acc0, 0u, stage, nv, t0, lo, ws);
-                else
-                    vote_tile<S, 4, false>(p, acc0, 0u, stage, nv, t0, lo, ws);
-                int before = is.n_list;                  // of the tiles before (no one adds to it now)
-                __syncthreads();
-                iter_list<S>(p, acc0, t0, lo, floor, nv > 255, list, q.cap_list, is);
-                __syncthreads();
-                while (is.n_list > q.cap_list) {
-                    // raise the floor until half the list is free, drop what
-                    // falls below it, and list the tile again
-                    for (int i = threadIdx.x; i < 64; i += NT)
-                        hist[i] = 0;
-                    __syncthreads();
-                    for (int i = threadIdx.x; i < q.cap_list; i += NT)
-                        atomicAdd(&hist[min((int)(list[i] >> shift), 63)], 1);
-                    __syncthreads();
-                    int n = 0, v = 64;
-                    while (v > 0 && n + hist[v - 1] <= q.cap_list / 2)
-                        n += hist[--v];
-                    floor = max(floor + 1, v);
-                    left = left || v > 63;               // too many to tell apart
-                    __syncthreads();
-                    if (warp == 0) {
-                        int m = 0;
-                        for (int i0 = 0; i0 < before; i0 += 32) {
-                            const uint32_t key = i0 + lane < before ? list[i0 + lane] : 0u;
-                            const unsigned mk = __ballot_sync(0xffffffffu, (int)(key >> shift) >= floor);
-                            if (mk >> lane & 1u)
-                                list[m + __popc(mk & lt)] = key;
-                            m += __popc(mk);
-                            __syncwarp();
-                        }
-                        if (lane == 0)
-                            is.n_list = m;
-                    }
-                    __syncthreads();
-                    before = is.n_list;
-                    __syncthreads();
-                    iter_list<S>(p, acc0, t0, lo, floor, false, list, q.cap_list, is);
-                    __syncthreads();
-                    if (left)
-                        break;
-                }
-                zero_tile<S>(p, tile);
-                __syncthreads();
-            }
-            if (nv > 255 && is.sum != (unsigned)nv * (unsigned)p.n_theta)
-                left = true;                             // a byte overflowed
-            if (left)
-                break;
-            // this thread's hits still unassigned: bit k for hit k NT + threadIdx.x
-            unsigned alive = 0u;
-            for (int k = 0; k * NT + (int)threadIdx.x < nv; ++k)
-                alive |= 1u << k;
-            // each warp keeps its share of the list, in place, and drops the
-            // bins that fall below the floor
-            const int first = found, share = (is.n_list + nw - 1) / nw;
-            uint32_t *mine = list + warp * share;
-            int n = max(min(share, is.n_list - warp * share), 0);
-            int n_tk = 0;
-            for (;;) {
-                // take the last track's votes from the listed bins; the best left
-                uint32_t best = 0u;
-                int kept = 0;
-                for (int i0 = 0; i0 < n; i0 += 32) {
-                    uint32_t key = i0 + lane < n ? mine[i0 + lane] : 0u;
-                    if (n_tk > 0) {
-                        // a hit is in the bin when its sum is within 2^K of the bin's
-                        // first (mod 2^32: the sums span less than 2^32 - 2^K)
-                        const unsigned at = ((1u << shift) - 1u) - (key & ((1u << shift) - 1u));
-                        const int t = min((int)(at >> p.bb), p.n_theta - 1);
-                        const unsigned c = (unsigned)__ldg(p.C + t), s = (unsigned)__ldg(p.S + t);
-                        const unsigned d = (unsigned)p.D - ((at & ((1u << p.bb) - 1u)) << p.K);
-                        const unsigned one = 1u << p.K;
-                        const int4 *pair = reinterpret_cast<const int4 *>(tk);
-                        unsigned off = 0u;
-#pragma unroll 4
-                        for (int x = 0; x < n_tk >> 1; ++x) {
-                            const int4 h = pair[x];
-                            off += (unsigned)h.x * c + (unsigned)h.y * s + d < one ? 1u : 0u;
-                            off += (unsigned)h.z * c + (unsigned)h.w * s + d < one ? 1u : 0u;
-                        }
-                        if (n_tk & 1) {
-                            const int2 h = tk[n_tk - 1];
-                            off += (unsigned)h.x * c + (unsigned)h.y * s + d < one ? 1u : 0u;
-                        }
-                        key -= off << shift;
-                    }
-                    const bool ok = i0 + lane < n && (int)(key >> shift) >= floor;
-                    const unsigned mk = __ballot_sync(0xffffffffu, ok);
-                    if (ok)
-                        mine[kept + __popc(mk & lt)] = key;
-                    kept += __popc(mk);
-                    best = max(best, ok ? key : 0u);
-                    __syncwarp();
-                }
-                n = kept;
-                best = __reduce_max_sync(0xffffffffu, best);
-                if (lane == 0)
-                    wtot[warp] = (int)best;
-                __syncthreads();
-                best = __reduce_max_sync(0xffffffffu, lane < nw ? (unsigned)wtot[lane] : 0u);
-                const int votes = (int)(best >> shift);
-                if (best == 0u || votes < floor || found == q.max_tracks)
-                    break;
-                const unsigned at = ((1u << shift) - 1u) - (best & ((1u << shift) - 1u));
-                const int bt = (int)(at >> p.bb), bb = (int)(at & ((1u << p.bb) - 1u));
-                const int c = __ldg(p.C + bt), s = __ldg(p.S + bt);
-                int &taken = is.taken[found & 1];
-                for (int k = 0; k * NT < nv; ++k) {
-                    const int i = k * NT + (int)threadIdx.x;
-                    bool take = false;
-                    int2 h = make_int2(0, 0);
-                    if (alive >> k & 1u) {
-                        h = stage[i];
-                        const int d = rho_bin(h.x, h.y, c, s, p.D, p.K) - bb;
-                        take = d <= p.tol && d >= -p.tol;
-                    }
-                    const unsigned m = __ballot_sync(0xffffffffu, take);
-                    if (m != 0u) {
-                        int base = 0;
-                        if (lane == 0)
-                            base = atomicAdd(&taken, __popc(m));
-                        base = __shfl_sync(0xffffffffu, base, 0);
-                        if (take) {
-                            alive &= ~(1u << k);
-                            tk[base + __popc(m & lt)] = h;
-                            p.hit_track[beg + sidx[i]] = found;
-                        }
-                    }
-                }
-                __syncthreads();
-                n_tk = taken;
-                if (threadIdx.x == 0) {
-                    q.tracks[(size_t)w * q.max_tracks + found] = make_int4(bt, bb, votes, n_tk);
-                    is.taken[(found + 1) & 1] = 0;
-                }
-                ++found;
-            }
-            if (floor == p.T || found == q.max_tracks)
-                break;
-            if (found == first) {
-                left = true;                             // more equal bins than the list holds
-                break;
-            }
-            // the hits left, in order, for the next list
-            int kept = 0;
-            __syncthreads();
-            for (int k = 0; k * NT < nv; ++k) {
-                const int i = k * NT + (int)threadIdx.x;
-                const bool keep = alive >> k & 1u;
-                const int2 h = keep ? stage[i] : make_int2(0, 0);
-                const uint16_t ix = keep ? sidx[i] : (uint16_t)0;
-                const unsigned m = __ballot_sync(0xffffffffu, keep);
-                if (lane == 0)
-                    wtot[warp] = __popc(m);
-                __syncthreads();
-                const int c = lane < nw ? wtot[lane] : 0;
-                const int pos = kept + (int)__reduce_add_sync(0xffffffffu, (unsigned)(lane < warp ? c : 0)) + __popc(m & lt);
-                if (keep) {
-                    stage[pos] = h;
-                    sidx[pos] = ix;
-                }
-                kept += (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
-                __syncthreads();
-            }
-            nv = kept;
-        }
-        if (threadIdx.x == 0) {
-            q.n_tracks[w] = left ? kIterLeft : found;
-            p.status[w] = ws.flags;
-        }
+        nv = kept;
     }
-    // the last CTA to finish resets the counters for the next launch
-    if (q.work && threadIdx.x == 0) {
-        __threadfence();
-        if (atomicAdd(q.work + 1, 1u) == gridDim.x - 1) {
-            atomicExch(q.work, 0u);
-            atomicExch(q.work + 1, 0u);
-            __threadfence();
-        }
+    if (threadIdx.x == 0) {
+        q.n_tracks[w] = left ? kIterLeft : found;
+        p.status[w] = ws.flags;
     }
 }
 
