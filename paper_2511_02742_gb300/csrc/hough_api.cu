@@ -209,8 +209,13 @@ int raise_smem_limit(const void *func, size_t bytes)
     return HOUGH_OK;
 }
 
+// Every failing call of a context returns through here.  The runtime's error of
+// an allocation or call that failed is taken off: the next call asks for the last
+// error after its launch, and would give this one back as its own.
 int fail(hough_ctx *ctx, int code)
 {
+    if (code == HOUGH_ERR_ALLOC || code == HOUGH_ERR_CUDA)
+        cudaGetLastError();
     if (ctx && code != HOUGH_OK)
         ctx->last_error = code;
     return code;
