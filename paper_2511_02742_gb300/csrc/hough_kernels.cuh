@@ -947,7 +947,12 @@ __device__ __forceinline__ int find_peaks(const KParams &p, const TileView &tv,
                 // histogram as it stands, not only at a merge (uneven heavy
                 // windows 427 -> 406 us; smaller windows lost 1%)
                 if constexpr (SUM) {
-                    const int stored = *reinterpret_cast<volatile int *>(&ws.n_buf);
+                    // one lane's look, for all: other warps are adding to it, and
+                    // the bound below is worked out by the whole warp
+                    int stored = 0;
+                    if (lane == 0)
+                        stored = *reinterpret_cast<volatile int *>(&ws.n_buf);
+                    stored = __shfl_sync(0xffffffffu, stored, 0);
                     if (stored - seen >= p.max_peaks) {
                         seen = stored;
                         vk = vote_bound(p, st, ws);
