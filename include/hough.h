@@ -469,7 +469,12 @@ int hough_set_launch(hough_ctx *ctx, const hough_launch *cfg);
 /*
  * Time every supported launch shape on this batch (iters runs each, CUDA
  * events on stream), keep the fastest in the context and return it in *best
- * (may be NULL).  Outputs are overwritten with the (identical) results.
+ * (may be NULL).  Where the library's own choice for the batch is as fast as
+ * the best of them (few windows: several CTAs per window), later calls are
+ * left to it, as after hough_set_launch with all fields 0, and *best is its
+ * first choice, as hough_get_launch gives it; a shape set with
+ * hough_set_launch holds for batches of every size.  Outputs are overwritten
+ * with the (identical) results.
  */
 int hough_autotune(hough_ctx *ctx, const hough_hits *hits, const int64_t *window_offsets,
                    int64_t n_windows, const hough_tracks *tracks_out, void *stream, int iters,

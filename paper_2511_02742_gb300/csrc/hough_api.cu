@@ -1590,8 +1590,22 @@ int hough_autotune(hough_ctx *ctx, const hough_hits *hits, const int64_t *window
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
         return fail(ctx, HOUGH_ERR_CUDA);
+    // one shape's time over iters calls; false when an event fails
+    auto time = [&](const hough_launch &l, bool automatic, float &ms) {
+        ms = 1e30f;
+        if (launch_find(ctx, hits, window_offsets, n_windows, tracks_out, s, c, l, automatic) != HOUGH_OK) {
+            cudaGetLastError();
+            return true;
+        }
+        cudaEventRecord(e0, s);
+        for (int i = 0; i < iters; ++i)
+            launch_find(ctx, hits, window_offsets, n_windows, tracks_out, s, c, l, automatic);
+        cudaEventRecord(e1, s);
+        return cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess;
+    };
     hough_launch chosen = ctx->launch;
-    float best_ms = 1e30f;
+    float best_ms = 1e30f, ms = 0.f;
+    bool ok = true;
     for (int threads : {128, 256, 512, 1024})
         for (int wr : {32, 64, 128})
             for (int cps : {1, 2, 3, 4})
@@ -1599,39 +1613,36 @@ int hough_autotune(hough_ctx *ctx, const hough_hits *hits, const int64_t *window
                     hough_launch req{threads, wr, hs, cps};
                     hough_launch l{};
                     size_t smem = 0;
-                    if (resolve_launch(ctx, req, l, smem) != HOUGH_OK)
+                    if (!ok || resolve_launch(ctx, req, l, smem) != HOUGH_OK)
                         continue;
                     if (cps > 1 && smem * cps > ctx->smem_optin)
                         continue;
-                    if (launch_find(ctx, hits, window_offsets, n_windows, tracks_out, s, c, l) !=
-                        HOUGH_OK) {
-                        cudaGetLastError();
-                        continue;
-                    }
-                    cudaEventRecord(e0, s);
-                    for (int i = 0; i < iters; ++i)
-                        launch_find(ctx, hits, window_offsets, n_windows, tracks_out, s, c, l);
-                    cudaEventRecord(e1, s);
-                    if (cudaEventSynchronize(e1) != cudaSuccess) {
-                        cudaEventDestroy(e0);
-                        cudaEventDestroy(e1);
-                        return fail(ctx, HOUGH_ERR_CUDA);
-                    }
-                    float ms = 0.f;
-                    cudaEventElapsedTime(&ms, e0, e1);
-                    if (ms < best_ms) {
+                    ok = time(l, false, ms);
+                    if (ok && ms < best_ms) {
                         best_ms = ms;
                         chosen = l;
                     }
                 }
+    // the library's own choice for the batch, which for few windows is none of
+    // those shapes (a cluster of CTAs per window): kept where it is not slower
+    hough_launch own{};
+    size_t own_smem = 0;
+    bool automatic = false;
+    if (ok && resolve_launch(ctx, hough_launch{}, own, own_smem) == HOUGH_OK) {
+        ok = time(launch_for(ctx, own, true, hits->n_hits, n_windows), true, ms);
+        automatic = ok && ms < 1e30f && ms <= best_ms;
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    ctx->launch = chosen;
-    ctx->auto_launch = false;
+    if (!ok)
+        return fail(ctx, HOUGH_ERR_CUDA);
+    ctx->launch = automatic ? own : chosen;
+    ctx->auto_launch = automatic;
     // leave the outputs holding the chosen shape's (identical) results
-    rc = launch_find(ctx, hits, window_offsets, n_windows, tracks_out, s, c, chosen);
+    rc = launch_find(ctx, hits, window_offsets, n_windows, tracks_out, s, c,
+                     launch_for(ctx, ctx->launch, automatic, hits->n_hits, n_windows), automatic);
     if (best)
-        *best = chosen;
+        *best = ctx->launch;
     return fail(ctx, rc);
 }
 
