@@ -531,11 +531,13 @@ int hough_find_noalloc(const hough_geometry *g, int n_theta, int n_rho,
  *     runs once over the batch, and each request's results are copied
  *     straight into its host buffers; the request then completes.
  * With n_slots > 1, requests that arrive while earlier batches are on the
- * GPU go into the next free slot (continuous batching), so their copies and
- * kernels overlap with the running ones: at once when the queue holds a window
- * per SM or more, else after up to 60 us, in which others may join them.  Device buffers and
- * pinned staging are allocated once, in hough_server_create, and stay
- * resident.  Each window's results are the same bits as hough_find gives it
+ * GPU go into the next free slot at once (continuous batching), so their
+ * copies and kernels overlap with the running ones.  Only while nobody looks
+ * at the results (no thread in wait or drain, four or more of them unread)
+ * do requests that follow one another within 60 us stay in the queue for up to
+ * 60 us, in which others may join them: until it holds a window per SM, or
+ * what a slot takes.  Device buffers and pinned staging are allocated once,
+ * in hough_server_create, and stay resident.  Each window's results are the same bits as hough_find gives it
  * alone: windows never interact.
  *
  * While a server exists it owns its context: make no other call on that

@@ -9,8 +9,8 @@
 //              requests (their results are in their buffers already);
 //   admit   -- a free slot and a non-empty queue: take requests, oldest
 //              first, while the slot's window and hit capacity allows
-//              (while another batch is on the GPU, fewer windows than SMs
-//              wait a moment for more),
+//              (few windows wait a moment for more while nobody looks at the
+//              results: hough_gather.h),
 //              write the batch's window offsets (rebased) into the slot's
 //              pinned staging, then on the slot's stream copy them and each
 //              request's hits in, launch the find kernel, copy the results
@@ -35,6 +35,7 @@
 #include <vector>
 
 #include "hough.h"
+#include "hough_gather.h"
 #include "hough_internal.h"
 
 namespace {
@@ -43,12 +44,6 @@ size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // How long an idle worker polls the queue before it sleeps.
 constexpr int64_t kIdleSpinNs = 2'000'000;
-
-// How long a request may wait for others while a batch is on the GPU and the
-// queue holds fewer windows than the GPU has SMs: requests that come one
-// after the other are then served by few batches with a window per SM, not by
-// one batch (ten copies and a launch) each.  About the time of such a batch.
-constexpr int64_t kGatherNs = 60'000;
 
 int64_t now_ns()
 {
@@ -93,6 +88,7 @@ struct Pending {
     hough_request req{};
     int64_t n_hits = 0;
     int64_t queued_ns = 0;
+    bool soon = false;               // the request before it came just before (Gather)
 };
 
 struct Slot {
@@ -129,6 +125,8 @@ struct hough_server {
     std::condition_variable cv_work;   // worker: a request was queued, or stop
     std::condition_variable cv_done;   // waiters: requests completed
     std::deque<Pending> queue;
+    Gather gather{0, 0, 0};
+    int waiting = 0;                     // threads in wait or drain
     std::unordered_set<uint64_t> live;                          // accepted, not yet delivered
     std::unordered_map<uint64_t, hough_request_result> done;    // completed, not yet delivered
     std::deque<uint64_t> done_order;                            // completion order (poll)
@@ -268,16 +266,27 @@ void complete_slot(hough_server *s, Slot &sl, int64_t t_done)
 // Whether the queued requests should wait for others (lock held).
 bool gather(const hough_server *s)
 {
+    if (s->stop || s->queue.empty())
+        return false;
     bool busy = false;
     for (const Slot &sl : s->slots)
         busy = busy || sl.busy;
-    if (!busy || s->stop || s->queue.empty())
-        return false;
-    int64_t windows = 0;
-    for (const Pending &p : s->queue)
-        if ((windows += p.req.n_windows) >= s->ctx->num_sms)
-            return false;
-    return now_ns() - s->queue.front().queued_ns < kGatherNs;
+    const Pending &p = s->queue.front();
+    return s->gather.hold(now_ns(), p.queued_ns, p.soon, busy, (int64_t)s->done.size(), s->waiting);
+}
+
+// Wait for `ready` (lock held), forever when timeout_ms < 0; false on a timeout.
+template <class Ready>
+bool wait_for(hough_server *s, std::unique_lock<std::mutex> &lk, int64_t timeout_ms, Ready ready)
+{
+    s->waiting += 1;
+    bool ok = true;
+    if (timeout_ms < 0)
+        s->cv_done.wait(lk, ready);
+    else
+        ok = s->cv_done.wait_for(lk, std::chrono::milliseconds(timeout_ms), ready);
+    s->waiting -= 1;
+    return ok;
 }
 
 void worker_loop(hough_server *s)
@@ -323,6 +332,7 @@ void worker_loop(hough_server *s)
                 s->queue.pop_front();
                 s->queued.fetch_sub(1, std::memory_order_release);
             }
+            s->gather.taken(sl.W, sl.H);
             sl.busy = true;
             s->in_flight += (int64_t)sl.reqs.size();
             s->st.batches += 1;
@@ -415,6 +425,7 @@ int hough_server_create(hough_ctx *ctx, const hough_server_config *cfg, hough_se
     }
     s->ctx = ctx;
     s->cfg = *cfg;
+    s->gather = Gather(ctx->num_sms, cfg->slot_windows, cfg->slot_hits);
     s->max_peaks = ctx->th.max_peaks;
     // the server's launch shape: as given, else chosen per batch: the
     // library's shapes for few windows (several CTAs per window, or large
@@ -524,6 +535,7 @@ int hough_server_submit(hough_server *s, const hough_request *req, uint64_t *tic
     if (p.req.arrival_ns == 0)
         p.req.arrival_ns = now_ns();
     p.queued_ns = now_ns();
+    p.soon = s->gather.queued(p.queued_ns, nw, nh);
     s->queue.push_back(p);
     s->queued.fetch_add(1, std::memory_order_release);
     s->live.insert(p.ticket);
@@ -541,10 +553,7 @@ int hough_server_wait(hough_server *s, uint64_t ticket, int64_t timeout_ms,
     std::unique_lock<std::mutex> lk(s->mu);
     if (!s->live.count(ticket))
         return HOUGH_ERR_INVALID_ARG;
-    auto ready = [&] { return s->done.count(ticket) != 0; };
-    if (timeout_ms < 0)
-        s->cv_done.wait(lk, ready);
-    else if (!s->cv_done.wait_for(lk, std::chrono::milliseconds(timeout_ms), ready))
+    if (!wait_for(s, lk, timeout_ms, [&] { return s->done.count(ticket) != 0; }))
         return HOUGH_ERR_TIMEOUT;
     if (res)
         *res = s->done[ticket];
@@ -578,12 +587,9 @@ int hough_server_drain(hough_server *s, int64_t timeout_ms)
     if (!s)
         return HOUGH_ERR_INVALID_ARG;
     std::unique_lock<std::mutex> lk(s->mu);
-    auto idle = [&] { return s->queue.empty() && s->in_flight == 0; };
-    if (timeout_ms < 0)
-        s->cv_done.wait(lk, idle);
-    else if (!s->cv_done.wait_for(lk, std::chrono::milliseconds(timeout_ms), idle))
-        return HOUGH_ERR_TIMEOUT;
-    return HOUGH_OK;
+    return wait_for(s, lk, timeout_ms, [&] { return s->queue.empty() && s->in_flight == 0; })
+               ? HOUGH_OK
+               : HOUGH_ERR_TIMEOUT;
 }
 
 int hough_server_get_stats(hough_server *s, hough_server_stats *out)
