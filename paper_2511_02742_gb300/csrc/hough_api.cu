@@ -913,6 +913,14 @@ int32_t g_noalloc_C[HOUGH_NOALLOC_MAX_THETA], g_noalloc_S[HOUGH_NOALLOC_MAX_THET
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
+void prepare_batch(hough_ctx *ctx, int64_t n_hits, int64_t n_windows)
+{
+    Prepared pr{};
+    if (prepare_find(ctx, n_windows, launch_for(ctx, ctx->launch, ctx->auto_launch, n_hits, n_windows),
+                     pr, ctx->auto_launch) != HOUGH_OK)
+        cudaGetLastError();
+}
+
 extern "C" {
 
 int hough_find_noalloc(const hough_geometry *g, int n_theta, int n_rho,

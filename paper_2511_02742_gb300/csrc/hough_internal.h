@@ -62,3 +62,8 @@ struct hough_ctx {
 // chosen from the batch's mean hits per window when `automatic`.
 hough_launch launch_for(const hough_ctx *ctx, const hough_launch &base, bool automatic,
                         int64_t n_hits, int64_t n_windows);
+
+// What the first hough_find of such a batch on this context sets up (loading the
+// kernel, raising its shared-memory limit, looking at its resources), without
+// launching it.  What fails here fails in the find, and is reported there.
+void prepare_batch(hough_ctx *ctx, int64_t n_hits, int64_t n_windows);

@@ -1,0 +1,36 @@
+"""The first request of each batch size costs what the next ones do: the kernels
+of all the library's shapes are set up when the server is created."""
+import os
+import subprocess
+
+import pytest
+
+from paper_2511_02742_gb300 import build, synth
+
+pytestmark = pytest.mark.gpu
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.mark.parametrize("n", [512, 1024])
+def test_first_request_of_each_size(hough, tmp_path, n):
+    """In a process of its own, since kernels stay set up in one.  Set up under
+    the request, 200 and 350 windows took 290 and 220 to 260 us longer.  The
+    server's very first request has more to wait for than its kernel."""
+    lib = build.build()
+    cuda = os.path.dirname(os.path.dirname(build.nvcc()))
+    exe = tmp_path / "first_request"
+    subprocess.run(["g++", "-std=c++17", "-O2", "-I", os.path.join(build.ROOT, "include"),
+                    "-I", os.path.join(cuda, "include"), os.path.join(HERE, "c", "first_request.cpp"),
+                    "-o", str(exe), "-L", os.path.dirname(lib), "-lhough",
+                    "-L", os.path.join(cuda, "lib64"), "-lcudart", "-lpthread",
+                    "-Wl,-rpath," + os.path.dirname(lib) + ":" + os.path.join(cuda, "lib64")],
+                   check=True)
+    geometry = tmp_path / "geometry.bin"
+    geometry.write_bytes(bytes(hough.make_geometry(synth.GEOMETRY)))
+    r = subprocess.run([str(exe), str(geometry), str(n)], check=True, timeout=120,
+                       capture_output=True, text=True)
+    rows = [[float(x) for x in line.split()] for line in r.stdout.splitlines()]
+    assert [row[0] for row in rows] == [1, 60, 200, 350, 700]
+    for w, first, later in rows:
+        if w > 60:
+            assert first < later + 120.0, (w, first, later)
