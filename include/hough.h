@@ -210,9 +210,15 @@ int hough_tables(const hough_geometry *g, int n_theta, int n_rho, int32_t *C, in
  * 0), n_rho - *nb) rounded down to a multiple of 4.  lo[k * T + i] (caller's
  * array of 3 T entries, T = ceil(n_theta / 32); entries past a width's last
  * tile are 0) receives tile i's first bin for counter width 2^k.  Contexts
- * use these for the fixed-point find (not for HOUGH_FLAG_FP64 or
- * hough_find_noalloc, whose tiles store every bin; with HOUGH_FLAG_EXPORT_ACC
- * *nb is rounded up to whole blocks of 32 bins and lo down to 8).
+ * use these for the fixed-point find, except that
+ *   - with HOUGH_FLAG_FP64 and in hough_find_noalloc tiles store every bin;
+ *   - with HOUGH_FLAG_EXPORT_ACC *nb is rounded up to whole blocks of 32 bins
+ *     and lo down to 8 (where n_rho is a multiple of 8, else 4);
+ *   - for n_theta <= 192 with 1 to 64 rows past a multiple of 128 (180 x 1000,
+ *     say) finds with 32 word rows have 64-row tiles at most, and their *nb is
+ *     the widest range over k = 0 and 1 only;
+ * and hough_accumulate, which shares the votes, stores whole blocks of 32 bins
+ * or all of them.
  * Errors: INVALID_ARG (null pointer, bad geometry or word_rows),
  * UNSUPPORTED_SHAPE (as hough_create).
  */

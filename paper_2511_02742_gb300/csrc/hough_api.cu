@@ -119,11 +119,54 @@ static void narrow_tiles(const hough_geometry *g, int nt, int nr, const int32_t 
 // fewer bins.  (180 x 1000: 6 votes a hit instead of 8, 708 bins a row instead
 // of 788, two CTAs per SM instead of one: 267 -> 206 us per 3001 windows.)  From
 // 256 rows on the longer tiles' fewer scans weigh more.
+static int find_pmax(int n_theta)
+{
+    const int r = n_theta % 128;
+    return n_theta <= 192 && r > 0 && r <= 64 ? 2 : 4;
+}
+
 static int find_pmax(const hough_ctx *ctx)
 {
-    const int r = ctx->n_theta % 128;
-    return !(ctx->th.flags & HOUGH_FLAG_FP64) && ctx->n_theta <= 192 && r > 0 && r <= 64 ? 2 : 4;
+    return ctx->th.flags & HOUGH_FLAG_FP64 ? 4 : find_pmax(ctx->n_theta);
 }
+
+// The narrowed tiles of a fixed-point context.  Bins stored per row, and the
+// first ones in lo, [table][log2 P][tile] with `stride` between rows of tiles:
+// tables 0 to 2 the find's for 32, 64 and 128 word rows, 3 hough_accumulate's,
+// 4 (if find_nb > 0) the find's own for 32 word rows where its tiles have two
+// counters a word at most.
+struct TileLayouts {
+    int nb[3], acc_nb, find_nb, stride;
+    std::vector<int32_t> lo;
+};
+
+static void tile_layouts(const hough_geometry *g, int nt, int nr, const int32_t *C, const int32_t *S,
+                         long long D, int K, bool exported, size_t smem_per_sm, TileLayouts &out)
+{
+    // with the export on, tiles of whole blocks of 32 bins that start on a
+    // 32-byte sector of the output
+    const int bins = exported ? 32 : 4, first = exported && nr % 8 == 0 ? 8 : 4;
+    out.stride = (nt + 31) / 32;
+    const size_t per = (size_t)3 * out.stride;
+    narrow_tiles(g, nt, nr, C, S, D, K, out.nb, out.lo, bins, first);
+    // hough_accumulate's: blocks of 32 bins, whole 128-byte lines of the
+    // output where its rows are; full-width tiles where three CTAs per SM
+    // hold them (their stores are then whole rows: 2000 windows of 142 hits
+    // at 512 x 512, 349 us narrowed, 343 us full-width)
+    std::vector<int32_t> lo(per, 0);
+    int nb[3] = {nr, 0, 0};
+    if (3 * (hk::tile_words(32, nr) * 4 + (size_t)hk::kAccStage * 8 + 2048) > smem_per_sm)
+        narrow_tiles(g, nt, nr, C, S, D, K, nb, lo, 32, nr % 32 == 0 ? 32 : 4);
+    out.acc_nb = nb[0];
+    out.lo.insert(out.lo.end(), lo.begin(), lo.begin() + per);
+    out.find_nb = 0;
+    if (find_pmax(nt) == 2) {
+        narrow_tiles(g, nt, nr, C, S, D, K, nb, lo, bins, first, 2);
+        out.find_nb = nb[0];
+        out.lo.insert(out.lo.end(), lo.begin(), lo.begin() + per);
+    }
+}
+
 
 // Bins a find tile stores per row for this word-row count.
 static int find_bins(const hough_ctx *ctx, int word_rows);
@@ -702,6 +745,29 @@ int hough_tile_bins(const hough_geometry *g, int n_theta, int n_rho, int word_ro
     return HOUGH_OK;
 }
 
+int hough_tiles_in_use(const hough_geometry *g, int n_theta, int n_rho, int use, int64_t smem_per_sm,
+                       int32_t *nb, int32_t *p_max, int32_t *lo)
+{
+    if (!geometry_ok(g) || !nb || !p_max || !lo || use < 0 || use > 2 || smem_per_sm < 0)
+        return HOUGH_ERR_INVALID_ARG;
+    if (n_theta < 1 || n_theta > HOUGH_MAX_THETA || n_rho < 4 || n_rho > HOUGH_MAX_RHO || n_rho % 4 != 0)
+        return HOUGH_ERR_UNSUPPORTED_SHAPE;
+    std::vector<int32_t> C(n_theta), S(n_theta);
+    int64_t D = 0;
+    int32_t K = 0;
+    const int rc = hough_tables(g, n_theta, n_rho, C.data(), S.data(), &D, &K);
+    if (rc != HOUGH_OK)
+        return rc;
+    TileLayouts t;
+    tile_layouts(g, n_theta, n_rho, C.data(), S.data(), D, K, use == 1, (size_t)smem_per_sm, t);
+    const int table = use == 2 ? 3 : t.find_nb > 0 ? 4 : 0;
+    *nb = table == 3 ? t.acc_nb : table == 4 ? t.find_nb : t.nb[0];
+    *p_max = table == 4 ? 2 : 4;
+    const size_t per = (size_t)3 * t.stride;
+    std::memcpy(lo, t.lo.data() + table * per, per * sizeof(int32_t));
+    return HOUGH_OK;
+}
+
 int hough_create(const hough_geometry *g, int n_theta, int n_rho, const hough_thresholds *th,
                  hough_ctx **out)
 {
@@ -760,33 +826,14 @@ int hough_create(const hough_geometry *g, int n_theta, int n_rho, const hough_th
     if (!(th->flags & HOUGH_FLAG_FP64)) {
         // narrowed tiles (the FP64 variant's bins come from another formula,
         // so its tiles keep every bin)
-        std::vector<int32_t> lo_all;
-        // with the export on, tiles of whole blocks of 32 bins that start on a
-        // 32-byte sector of the output
-        const bool exported = (th->flags & HOUGH_FLAG_EXPORT_ACC) != 0;
-        narrow_tiles(&ctx->g, ctx->n_theta, ctx->n_rho, ctx->C.data(), ctx->S.data(), ctx->D,
-                     ctx->K, ctx->tile_nb, lo_all, exported ? 32 : 4,
-                     exported && ctx->n_rho % 8 == 0 ? 8 : 4);
-        ctx->lo_stride = (ctx->n_theta + 31) / 32;
-        // hough_accumulate's: blocks of 32 bins, whole 128-byte lines of the
-        // output where its rows are; full-width tiles where three CTAs per SM
-        // hold them (their stores are then whole rows: 2000 windows of 142 hits
-        // at 512 x 512, 349 us narrowed, 343 us full-width)
-        std::vector<int32_t> lo_acc((size_t)3 * ctx->lo_stride, 0);
-        int nb_acc[3] = {ctx->n_rho, 0, 0};
-        if (3 * (hk::tile_words(32, ctx->n_rho) * 4 + (size_t)hk::kAccStage * 8 + 2048) > ctx->smem_per_sm)
-            narrow_tiles(&ctx->g, ctx->n_theta, ctx->n_rho, ctx->C.data(), ctx->S.data(), ctx->D,
-                         ctx->K, nb_acc, lo_acc, 32, ctx->n_rho % 32 == 0 ? 32 : 4);
-        ctx->acc_nb = nb_acc[0];
-        lo_all.insert(lo_all.end(), lo_acc.begin(), lo_acc.begin() + 3 * ctx->lo_stride);
-        if (find_pmax(ctx) == 2) {
-            int nb_find[3];
-            narrow_tiles(&ctx->g, ctx->n_theta, ctx->n_rho, ctx->C.data(), ctx->S.data(), ctx->D,
-                         ctx->K, nb_find, lo_acc, exported ? 32 : 4,
-                         exported && ctx->n_rho % 8 == 0 ? 8 : 4, 2);
-            ctx->find_nb = nb_find[0];
-            lo_all.insert(lo_all.end(), lo_acc.begin(), lo_acc.begin() + 3 * ctx->lo_stride);
-        }
+        TileLayouts tiles;
+        tile_layouts(&ctx->g, ctx->n_theta, ctx->n_rho, ctx->C.data(), ctx->S.data(), ctx->D, ctx->K,
+                     (th->flags & HOUGH_FLAG_EXPORT_ACC) != 0, ctx->smem_per_sm, tiles);
+        std::memcpy(ctx->tile_nb, tiles.nb, sizeof ctx->tile_nb);
+        ctx->acc_nb = tiles.acc_nb;
+        ctx->find_nb = tiles.find_nb;
+        ctx->lo_stride = tiles.stride;
+        const std::vector<int32_t> &lo_all = tiles.lo;
         if (cudaMalloc(&ctx->d_lo, sizeof(int32_t) * lo_all.size()) != cudaSuccess) {
             hough_destroy(ctx);
             return HOUGH_ERR_ALLOC;

@@ -63,6 +63,14 @@ struct hough_ctx {
 hough_launch launch_for(const hough_ctx *ctx, const hough_launch &base, bool automatic,
                         int64_t n_hits, int64_t n_windows);
 
+// The narrowed tiles that a context uses with 32 word rows, host only, for tests:
+// use 0 the find's, 1 with HOUGH_FLAG_EXPORT_ACC, 2 hough_accumulate's, on a
+// device with this much shared memory per SM.  *nb bins per row, *p_max counters
+// per word at most, lo[k * T + i] the first bin of tile i with 2^k counters per
+// word, T = ceil(n_theta / 32).
+extern "C" int hough_tiles_in_use(const hough_geometry *g, int n_theta, int n_rho, int use,
+                                  int64_t smem_per_sm, int32_t *nb, int32_t *p_max, int32_t *lo);
+
 // What the first hough_find of such a batch on this context sets up (loading the
 // kernel, raising its shared-memory limit, looking at its resources), without
 // launching it.  What fails here fails in the find, and is reported there.
