@@ -194,7 +194,7 @@ static int device_limits(hough_ctx *ctx, int dev)
             cudaSuccess)
         return HOUGH_ERR_CUDA;
     // the kernel's static shared scalars share the per-block limit
-    ctx->smem_optin = (size_t)smem_optin - 128;
+    ctx->smem_optin = (size_t)smem_optin - hk::kStaticSmem;
     ctx->smem_per_sm = (size_t)smem_sm;
     return HOUGH_OK;
 }
@@ -308,7 +308,8 @@ size_t find_smem(const hough_ctx *ctx, int word_rows, int hit_stage, int threads
 
 // Whether `ctas` CTAs of this much dynamic shared memory fit on an SM: per
 // CTA the SM also reserves 1 KB and holds the kernel's static shared
-// variables (kStaticSmemReserve covers them).
+// variables (kStaticSmemReserve covers them; hk::kStaticSmem bounds those of the
+// cluster kernels, which are not looked at here, when they are compiled).
 bool smem_fits(const hough_ctx *ctx, size_t smem, int ctas)
 {
     return smem <= std::min(ctx->smem_optin,
@@ -1218,7 +1219,7 @@ int hough_find_iterative(hough_ctx *ctx, const hough_hits *hits, const int64_t *
     hk::IterParams q{};
     int ctas = 4;
     for (; ctas >= 1; --ctas) {
-        const size_t share = std::min(ctx->smem_optin + 128 - fa.sharedSizeBytes,
+        const size_t share = std::min(ctx->smem_optin + hk::kStaticSmem - fa.sharedSizeBytes,
                                       ctx->smem_per_sm / (size_t)ctas - 1024 - fa.sharedSizeBytes);
         const size_t fixed = hk::iter_smem_bytes(nb, cap_hits, 0);
         if (fixed + 1536 * 4 <= share) {
@@ -1230,8 +1231,8 @@ int hough_find_iterative(hough_ctx *ctx, const hough_hits *hits, const int64_t *
     // the rest: 512 threads, tiles of 32 word rows beside the stage of hits and
     // the kernel's static shared variables (small tiles let more of them be
     // skipped once their count bound falls; 64 or 128 word rows were slower)
-    const size_t room = ctx->smem_optin + 128 > fb.sharedSizeBytes
-                            ? ctx->smem_optin + 128 - fb.sharedSizeBytes : 0;
+    const size_t room = ctx->smem_optin + hk::kStaticSmem > fb.sharedSizeBytes
+                            ? ctx->smem_optin + hk::kStaticSmem - fb.sharedSizeBytes : 0;
     const size_t smem_tiles = (size_t)32 * nb * 4 + (size_t)HOUGH_ITER_MAX_HITS * 12;
     if (smem_tiles > room || ctas < 1)
         return fail(ctx, HOUGH_ERR_UNSUPPORTED_SHAPE);

@@ -1553,6 +1553,12 @@ struct SplitOut {
     int overflow;        // a byte counter overflowed (SUM)
 };
 
+// The find kernels' static shared variables, beside the dynamic shared memory that
+// the host sizes to the device's limits less kStaticSmem.
+constexpr size_t kStaticSmem = 128;
+static_assert(sizeof(WinScalars) <= kStaticSmem && sizeof(WinScalars) + sizeof(SplitOut) <= kStaticSmem,
+              "static shared memory of the find kernels");
+
 __device__ __forceinline__ void cluster_sync()
 {
     asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
