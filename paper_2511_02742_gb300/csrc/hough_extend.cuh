@@ -146,12 +146,12 @@ __device__ __forceinline__ void extend_body(const ExtParams &q)
                 const int ht = p.hit_track[beg + i];
                 int v = -1;
                 if (ok && ht != -2) {
+                    // an address whose phi wraps into the box (and would be no
+                    // index) counts as its encoded phi does
                     if (p.box.raw)
                         v = __ldg(p.a + beg + i);
-                    else if (phi % vstep == 0)
-                        v = phi / vstep;
-                    if (v >= nv)
-                        v = -1;
+                    if ((unsigned)v >= (unsigned)nv)
+                        v = phi % vstep == 0 ? phi / vstep : -1;
                 }
                 zs[i] = z;
                 vs[i] = (int16_t)v;
