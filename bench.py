@@ -1110,7 +1110,7 @@ def run_ours(args):
                          if smem_peak["value"] else None,
                          "traffic": traffic[0], "traffic_source": traffic[1],
                          "peak_source": smem_peak["source"],
-                         "peak_red_no_return": smem_peak.get("red_no_return_gops"),
+                         "peak_atom_returned": smem_peak.get("returned_gops"),
                          "algorithmic": f"{votes} shared-memory vote atomics per launch "
                                         f"(valid hits x n_theta)",
                          "hbm": {"achieved_gbs": round(algo_bytes / (ms * 1e-3) / 1e9, 2),
@@ -1182,7 +1182,8 @@ def _smem_atomic_peak_gops(args):
     """Shared-memory atomic throughput measured by the bench-side probe
     (conflict-free 32-bit adds, all SMs), or the unit-count figure if the probe
     is off.  The ceiling is the form the vote loop issues: red.shared.add, with
-    no returned value."""
+    no returned value; the rate of atom.shared.add with the old value consumed
+    is given beside it."""
     nominal = 152 * 32 * 2.070   # SMs x banks x GHz: one 32-lane wavefront per clock per SM
     if args.no_probe:
         return {"value": round(nominal, 1), "source": "nominal: 152 SMs x 32 banks x 2.07 GHz"}
@@ -1192,7 +1193,7 @@ def _smem_atomic_peak_gops(args):
         return {"value": round(r, 1),
                 "source": "measured: conflict-free red.shared.add.u32 with no returned value "
                           "(the vote loop's op), bench_probe",
-                "red_no_return_gops": round(r, 1)}
+                "returned_gops": round(bench_probe.smem_atomic_gops("atom"), 1)}
     except Exception as e:  # pragma: no cover
         return {"value": round(nominal, 1), "source": f"nominal (probe failed: {e})"}
 

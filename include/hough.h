@@ -256,8 +256,12 @@ int hough_encode(hough_ctx *ctx, const int32_t *vane, const int32_t *strip, int6
  * (no memory outside [0, n_hits) is touched).  Windows must not overlap: two
  * windows sharing a hit write the same hit_track/track_hits slots.
  * Asynchronous on stream; results are identical for every launch shape,
- * stream and batch.
- * Errors: INVALID_ARG (bad pointers/sizes), CUDA (launch failed).
+ * stream and batch.  A call on a stream that captures a graph keeps the
+ * scheduling counter of that stream: no other find of the context on it, and
+ * no other graph captured on it, may run beside the graph (hough_plan_create
+ * captures with a counter of its own).
+ * Errors: INVALID_ARG (bad pointers/sizes), ALLOC (the first call on a stream
+ * allocates its counter), CUDA (launch failed).
  */
 int hough_find(hough_ctx *ctx, const hough_hits *hits, const int64_t *window_offsets,
                int64_t n_windows, const hough_tracks *tracks_out, void *stream);
@@ -390,9 +394,9 @@ int hough_find_iterative(hough_ctx *ctx, const hough_hits *hits, const int64_t *
  *                  claimed, ext_hits in index order), or HOUGH_WIN_BAD_OFFSETS
  *                  when the window's offsets are out of order or beyond
  *                  n_hits (its outputs are not written).
- * Asynchronous on stream; three launches.  Errors: INVALID_ARG (NULL
- * pointer, tol_z out of range), UNSUPPORTED_SHAPE (n_vanes outside
- * 3..HOUGH_EXT_MAX_VANES), CUDA.
+ * Asynchronous on stream; three launches, one for up to four windows per SM.
+ * Errors: INVALID_ARG (NULL pointer, tol_z out of range), UNSUPPORTED_SHAPE
+ * (n_vanes outside 3..HOUGH_EXT_MAX_VANES), CUDA.
  */
 #define HOUGH_EXT_MAX_HITS 4096
 #define HOUGH_EXT_MAX_VANES 256

@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(512, 1) iterative_tiles_kernel(IterParams q)
                     kept += tot;
                     __syncthreads();
                 }
-    #pragma unroll
+#pragma unroll
                 for (int d = 16; d > 0; d >>= 1)
                     mine += __shfl_xor_sync(0xffffffffu, mine, d);
                 if (lane == 0 && mine)
@@ -321,12 +321,12 @@ __global__ void __launch_bounds__(512, 1) iterative_tiles_kernel(IterParams q)
                 nv = kept;
                 ++found;
                 __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            q.n_tracks[w] = found;
-            p.status[w] = flags | ws.flags;
-        }
-        __syncthreads();
+            }
+            if (threadIdx.x == 0) {
+                q.n_tracks[w] = found;
+                p.status[w] = flags | ws.flags;
+            }
+            __syncthreads();
         }
     }
 }
@@ -543,7 +543,9 @@ __device__ __forceinline__ void iter_body(const IterParams &q)
                 uint32_t key = i0 + lane < n ? mine[i0 + lane] : 0u;
                 if (n_tk > 0) {
                     // a hit is in the bin when its sum is within 2^K of the bin's
-                    // first (mod 2^32: the sums span less than 2^32 - 2^K)
+                    // first.  Exact mod 2^32 for any geometry: sums are int32, and a
+                    // listed bin holds some, so it is [m 2^K, (m + 1) 2^K) inside
+                    // int32's range (2^K divides 2^31), which no other sum meets
                     const unsigned at = ((1u << shift) - 1u) - (key & ((1u << shift) - 1u));
                     const int t = min((int)(at >> p.bb), p.n_theta - 1);
                     const unsigned c = (unsigned)__ldg(p.C + t), s = (unsigned)__ldg(p.S + t);
